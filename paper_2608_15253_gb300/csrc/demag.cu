@@ -21,9 +21,11 @@
 
 #include "common.cuh"
 #include "ctx.h"
+#include "conv_lane.cuh"
 #include "fft_ct.cuh"
 #include "fft_direct.cuh"
 #include "fft_rt.cuh"
+#include "lane.h"
 
 namespace mm {
 
@@ -582,11 +584,12 @@ __device__ __forceinline__ void tensor_multiply(const ColArgs<T>& a, cplx<T>* sm
     __syncthreads();
 }
 
-template <typename T, int MODE, int LT>  // MODE: +1 forward, -1 inverse, 0 convolution
+// any length 2^a 3^b (those without a kernel of their own): runtime plan
+template <typename T, int MODE>  // MODE: +1 forward, -1 inverse, 0 convolution
 __global__ void __launch_bounds__(512) fft_col_kernel(ColArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* sm = reinterpret_cast<cplx<T>*>(smem_raw);
-    const int L = LT > 0 ? LT : a.L;
+    const int L = a.L;
     const int pitch = L + 1;
     const int kx0 = blockIdx.x * a.TK;
     const long long obase = (long long)blockIdx.y * a.other_stride;
@@ -604,18 +607,11 @@ __global__ void __launch_bounds__(512) fft_col_kernel(ColArgs<T> a) {
         }
     }
     __syncthreads();
-    constexpr int NT = LT >= 512 ? 512 : 256;
-    if constexpr (LT > 0) {
-        if (MODE >= 0) ct_fft<T, 1, LT, LT + 1, NT, kMaxV>(sm, nl, a.n_in, a.tw, 1);
-        else ct_fft<T, -1, LT, LT + 1, NT, kMaxV>(sm, nl, a.n_in, a.tw, 1);
-    } else {
-        if (MODE >= 0) fft_lines<T, 1>(sm, nl, pitch, a.plan, a.n_in, a.tw, 1);
-        else fft_lines<T, -1>(sm, nl, pitch, a.plan, a.n_in, a.tw, 1);
-    }
+    if (MODE >= 0) fft_lines<T, 1>(sm, nl, pitch, a.plan, a.n_in, a.tw, 1);
+    else fft_lines<T, -1>(sm, nl, pitch, a.plan, a.n_in, a.tw, 1);
     if (MODE == 0) {
         tensor_multiply<T>(a, sm, pitch, kx0, L, tks);
-        if constexpr (LT > 0) ct_fft<T, -1, LT, LT + 1, NT, kMaxV>(sm, nl, LT, a.tw, 1);
-        else fft_lines<T, -1>(sm, nl, pitch, a.plan, L, a.tw, 1);
+        fft_lines<T, -1>(sm, nl, pitch, a.plan, L, a.tw, 1);
     }
     for (int c = 0; c < a.nc; ++c) {
         cplx<T>* dst = a.base + c * a.comp_stride + obase + kx0;
@@ -629,40 +625,7 @@ __global__ void __launch_bounds__(512) fft_col_kernel(ColArgs<T> a) {
 // ---------------------------------------------------------------------------
 // FP32 3-D fast paths
 // ---------------------------------------------------------------------------
-// Y passes: TK = 16 columns per CTA taken from the flattened (component, z,
-// kx) column list, so no CTA is left with a ragged handful of columns; the
-// first Stockham pass reads global memory straight into registers and the
-// last one writes its outputs straight back (128-byte row segments).
-template <typename T>
-struct YArgs {
-    cplx<T>* base;        // spectrum [3][nz][Py][Wk]
-    long long plane;      // Py * Wk: between consecutive (component, z) planes
-    int Kx, Wk;
-    int ncols;            // 3 * nz * Kx
-    int n_in, n_out;
-    const cplx<T>* tw;    // exp(-2 pi i q / Py)
-};
-
-// Columns per CTA and threads: 16 columns, except at L >= 1024 where 8
-// columns of 256 threads (64 KB of shared memory) let three CTAs share an SM.
-__host__ __device__ constexpr int y_direct_tk(int L) { return L >= 1024 ? 8 : 16; }
-__host__ __device__ constexpr int y_direct_threads(int L) { return L >= 1024 ? 256 : L >= 512 ? 512 : 256; }
-
-template <typename T, int DIR, int L>
-__global__ void __launch_bounds__(y_direct_threads(L)) fft_y_direct_kernel(YArgs<T> a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    cplx<T>* sm = reinterpret_cast<cplx<T>*>(smem_raw);
-    constexpr int TK = y_direct_tk(L);
-    const int col = blockIdx.x * TK + (int)(threadIdx.x % TK);
-    long long gcol = -1;
-    if (col < a.ncols) {
-        const int q = col / a.Kx, kx = col - q * a.Kx;
-        gcol = (long long)q * a.plane + kx;
-    }
-    cd_fft<T, DIR, L, y_direct_threads(L), TK>(sm, a.base, a.base, gcol, a.Wk, a.n_in, a.n_out, a.tw);
-}
-
-// Middle (z) pass for Pz a power of two <= 32: one thread per (component,
+// Middle (z) pass for Pz a power of two <= 16: one thread per (component,
 // column) keeps its whole z line in registers.  Forward by decimation in
 // frequency (bit-reversed spectrum), the three components exchanged once
 // through shared memory for H^ = K^ M^ (row c of the symmetric tensor), then
@@ -1022,7 +985,6 @@ static int col_tk(int L, int nc) {
     X(16) X(32) X(48) X(64) X(81) X(96) X(108) X(128) X(162) X(192) X(216) X(256) X(324) X(432) X(512) X(1024)
 
 template <typename T> using XKern = void (*)(XArgs<T>);
-template <typename T> using CKern = void (*)(ColArgs<T>);
 
 template <typename T>
 static XKern<T> x_kernel(bool fwd, int Lh) {
@@ -1035,19 +997,6 @@ static XKern<T> x_kernel(bool fwd, int Lh) {
         }
     }
     return fwd ? fft_x_r2c_kernel<T, 0> : fft_x_c2r_kernel<T, 0>;
-}
-
-template <typename T, int MODE>
-static CKern<T> col_kernel(int L) {
-    if constexpr (sizeof(T) == 4) {
-        switch (L) {
-#define MM_CASE(n) case n: return fft_col_kernel<T, MODE, n>;
-            MM_CT_LENGTHS(MM_CASE)
-#undef MM_CASE
-            default: break;
-        }
-    }
-    return fft_col_kernel<T, MODE, 0>;
 }
 
 // lanes per row of the one-row-per-warp kernels (warp_group of the length)
@@ -1106,29 +1055,18 @@ static XKern<float> x_stage_kernel(int s, int Lh) {
 #undef MM_ST
 }
 
-using YKern = void (*)(YArgs<float>);
 using ZKern = void (*)(ZArgs<float>);
-
-static YKern y_direct_kernel(bool fwd, int L) {
-    switch (L) {
-#define MM_CASE(n) case n: return fwd ? fft_y_direct_kernel<float, 1, n> : fft_y_direct_kernel<float, -1, n>;
-        MM_CT_LENGTHS(MM_CASE)
-#undef MM_CASE
-        default: return nullptr;
-    }
-}
 
 // half: nz <= Pz/2 (the zero-padded upper half of every z line is known)
 static ZKern zconv_reg_kernel(int L, bool half) {
     switch (L) {
 #define MM_CASE(n) case n: return half ? fft_zconv_reg_kernel<float, n, true> : fft_zconv_reg_kernel<float, n, false>;
-        MM_CASE(4) MM_CASE(8) MM_CASE(16) MM_CASE(32)
+        MM_CASE(4) MM_CASE(8) MM_CASE(16)
 #undef MM_CASE
         default: return nullptr;
     }
 }
 
-static size_t y_direct_smem(int L) { return (size_t)L * y_direct_tk(L) * sizeof(cplx<float>); }
 static size_t zconv_reg_smem(int L) { return (size_t)(L + 3 * L * kZT) * sizeof(cplx<float>); }
 
 template <typename T>
@@ -1224,21 +1162,114 @@ static void launch_col(mm_ctx* c, ColArgs<T> a, int n_other, const char* name, d
     const size_t smem = (size_t)a.nc * a.TK * (a.L + 1) * sizeof(cplx<T>);
     dim3 grid((a.Kx + a.TK - 1) / a.TK, n_other);
     LaunchScope ls(c, name, bytes);
-    col_kernel<T, MODE>(a.L)<<<grid, thr, smem, c->stream>>>(a);
+    fft_col_kernel<T, MODE><<<grid, thr, smem, c->stream>>>(a);
 }
 
-static void launch_y_direct(mm_ctx* c, bool fwd, cplx<float>* S, long long plane, int n_in, int n_out,
-                            const char* name, double bytes) {
-    const DemagPlan& d = c->dm;
-    YArgs<float> a{};
-    a.base = S; a.plane = plane; a.Kx = d.Kx; a.Wk = d.Wk;
-    a.ncols = 3 * c->grid.nz * d.Kx;
-    a.n_in = n_in; a.n_out = n_out;
-    a.tw = (const cplx<float>*)d.tw_y;
+// One column pass by its lane kernel: the CTAs of `sides` tiles of columns, or
+// as many persistent CTAs as fit.
+template <typename T>
+static void launch_lane(mm_ctx* c, const LaneKern<T>& k, const LaneArgs<T>& a, int sides, const char* name,
+                        double bytes) {
+    const int tiles = (a.n_cols + k.cols - 1) / k.cols;
+    int grid = tiles * sides;
+    if (k.persistent) {
+        int occ = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k.kern, k.threads, k.smem);
+        grid = std::min(tiles, std::max(1, occ) * sm_count());
+    }
     LaunchScope ls(c, name, bytes);
-    const int tk = y_direct_tk(d.Py);
-    y_direct_kernel(fwd, d.Py)<<<(unsigned)((a.ncols + tk - 1) / tk), y_direct_threads(d.Py), y_direct_smem(d.Py),
-                                 c->stream>>>(a);
+    k.kern<<<grid, k.threads, k.smem, c->stream>>>(a);
+}
+
+// Y pass of the spectrum [3][nz][Py][Wk]; false if the length has no kernel.
+template <typename T>
+static bool launch_lane_y(mm_ctx* c, bool fwd, cplx<T>* S, const char* name, double bytes) {
+    const DemagPlan& d = c->dm;
+    const LaneKern<T> k = lane_col<T>(d.Py, fwd);
+    if (!k.kern) return false;
+    LaneArgs<T> a{};
+    a.base = S;
+    a.line_stride = d.Wk;
+    a.o_stride = (long long)d.Py * d.Wk;
+    a.Wk = d.Wk; a.Kx = d.Kx;
+    a.n_cols = 3 * c->grid.nz * d.Wk;
+    a.n_in = fwd ? c->grid.ny : d.Py;
+    a.n_out = fwd ? d.Py : c->grid.ny;
+    a.tw = (const cplx<T>*)d.tw_y;
+    launch_lane<T>(c, k, a, 1, name, bytes);
+    return true;
+}
+
+// 3-D middle pass along z; false if the length has no kernel.
+template <typename T>
+static bool launch_lane_z(mm_ctx* c, cplx<T>* S, double bytes) {
+    const DemagPlan& d = c->dm;
+    const LaneKern<T> k = lane_conv3<T>(d.Pz);
+    if (!k.kern) return false;
+    LaneArgs<T> a{};
+    const long long plane = (long long)d.Py * d.Wk, Ky = d.Py / 2 + 1, Kz = d.Pz / 2 + 1;
+    a.base = S;
+    a.comp_stride = c->grid.nz * plane;
+    a.line_stride = plane;
+    a.o_stride = d.Wk;
+    a.Wk = d.Wk; a.Kx = d.Kx;
+    a.n_o = d.Py;
+    a.n_cols = (int)(Ky * d.Wk);
+    a.n_in = a.n_out = c->grid.nz;
+    a.khat = (const T*)d.khat;
+    a.kc = Kz * Ky * d.Wk; a.kk = Ky * d.Wk; a.ko = d.Wk;
+    a.tw = (const cplx<T>*)d.tw_z;
+    launch_lane<T>(c, k, a, 2, "fft_conv", bytes);
+    return true;
+}
+
+// 2-D middle pass along y over n_planes films of the plan's size (plane r,
+// component q at S + r plane_stride + q comp_stride); false if the length has
+// no kernel.  A few hundred columns take the kernel with the shortest chain
+// per CTA (every component its own threads); once the other's wider CTAs
+// cover the SMs twice it does less work per column (96^2: 41 against 49 us
+// over 213 films; 512^2, one film: the other way round).
+template <typename T>
+static bool launch_lane_films(mm_ctx* c, const DemagPlan& p, cplx<T>* S, int ny, long long comp_stride,
+                              long long plane_stride, int n_planes, const char* name, double bytes) {
+    LaneKern<T> k = lane_films<T>(p.Py);
+    if (!k.kern || (long long)n_planes * p.Wk < 2LL * sm_count() * k.cols) {
+        const LaneKern<T> f = lane_film<T>(p.Py);
+        if (f.kern) k = f;
+    }
+    if (!k.kern) return false;
+    LaneArgs<T> a{};
+    a.comp_stride = comp_stride;
+    a.line_stride = p.Wk;
+    a.o_stride = plane_stride;
+    a.Wk = p.Wk; a.Kx = p.Kx;
+    a.n_in = a.n_out = ny;
+    a.khat = (const T*)p.khat;
+    a.kc = (long long)(p.Py / 2 + 1) * p.Wk;
+    a.kk = p.Wk;
+    a.tw = (const cplx<T>*)p.tw_y;
+    const int most = std::max(1, (1 << 30) / p.Wk);      // planes whose columns an int can count
+    for (int r = 0; r < n_planes; r += most) {
+        a.base = S + r * plane_stride;
+        a.n_o = std::min(most, n_planes - r);
+        a.n_cols = a.n_o * p.Wk;
+        launch_lane<T>(c, k, a, 1, name, bytes * a.n_o / n_planes);
+    }
+    return true;
+}
+
+// Opt the lane kernels of a plan into their shared memory (outside any capture).
+template <typename T>
+static cudaError_t lane_attributes(const DemagPlan& d, bool three_d) {
+    const LaneKern<T> ks[] = {three_d ? lane_col<T>(d.Py, true) : lane_film<T>(d.Py),
+                              three_d ? lane_col<T>(d.Py, false) : lane_films<T>(d.Py),
+                              three_d ? lane_conv3<T>(d.Pz) : LaneKern<T>{}};
+    for (const LaneKern<T>& k : ks)
+        if (k.kern) {
+            const cudaError_t e = cudaFuncSetAttribute(k.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
 }
 
 // c2r = false: every pass but the inverse X pass (which the fused inverse-X +
@@ -1257,20 +1288,14 @@ static void demag_apply_t(mm_ctx* c, const T* m, T* Hd, int stage = 0, bool c2r 
     launch_x<T>(c, true, m, nullptr, S, 3 * nz * ny, ny, d.PyA, nx, nx, d.Lh, (const cplx<T>*)d.tw_x, true, N,
                 stage);
     const bool three_d = nz > 1;
-    const bool fast_y = sizeof(T) == 4 && three_d && y_direct_kernel(true, d.Py) != nullptr;
-    const bool fast_z = sizeof(T) == 4 && three_d && zconv_reg_kernel(d.Pz, false) != nullptr;
-    const bool split_y = sizeof(T) == 4 && three_d && ysplit_supported(d.Py);
-    if (three_d && d.Py > 1 && split_y) {
-        ysplit_launch(c, true, S, nz, d.Py, d.Kx, d.Wk, ny, d.Py, "fft_y_fwd", 3.0 * nz * d.Kx * (ny + d.Py) * cplxb);
-    } else if (three_d && d.Py > 1 && fast_y) {
-        launch_y_direct(c, true, (cplx<float>*)S, plane, ny, d.Py, "fft_y_fwd",
-                        3.0 * nz * d.Kx * (ny + d.Py) * cplxb);
-    } else if (three_d && d.Py > 1) {
+    const bool reg_z = sizeof(T) == 4 && three_d && zconv_reg_kernel(d.Pz, false) != nullptr;
+    const double ybytes = 3.0 * nz * d.Kx * (ny + d.Py) * cplxb;
+    if (three_d && d.Py > 1 && !launch_lane_y<T>(c, true, S, "fft_y_fwd", ybytes)) {
         ColArgs<T> a{};
         a.base = S; a.comp_stride = comp; a.line_stride = d.Wk; a.other_stride = plane;
         a.nc = 3; a.Kx = d.Kx; a.L = d.Py; a.n_in = ny; a.n_out = d.Py;
         a.tw = (const cplx<T>*)d.tw_y;
-        launch_col<T, 1>(c, a, nz, "fft_y_fwd", 3.0 * nz * d.Kx * (ny + d.Py) * cplxb);
+        launch_col<T, 1>(c, a, nz, "fft_y_fwd", ybytes);
     }
     {
         ColArgs<T> a{};
@@ -1279,7 +1304,9 @@ static void demag_apply_t(mm_ctx* c, const T* m, T* Hd, int stage = 0, bool c2r 
         a.ncomp = d.ncomp;
         const long long Ky = d.Py / 2 + 1, Kz = d.Pz / 2 + 1;
         a.kc_stride = Kz * Ky * d.Wk;
-        if (three_d && fast_z) {
+        const double zbytes = 3.0 * d.Py * d.Kx * 2 * nz * cplxb + (double)d.ncomp * Kz * Ky * d.Kx * realb;
+        const double fbytes = 3.0 * d.Kx * 2 * ny * cplxb + (double)d.ncomp * Ky * d.Kx * realb;
+        if (reg_z) {
             ZArgs<float> z{};
             z.base = (cplx<float>*)S; z.comp_stride = comp; z.plane = plane;
             z.nz = nz; z.Py = d.Py; z.Kx = d.Kx; z.Wk = d.Wk;
@@ -1287,45 +1314,33 @@ static void demag_apply_t(mm_ctx* c, const T* m, T* Hd, int stage = 0, bool c2r 
             z.khat = (const float*)d.khat;
             z.kc_stride = a.kc_stride; z.kk_stride = Ky * d.Wk;
             const long long cols = (long long)d.Py * d.Wk;
-            LaunchScope ls(c, "fft_conv",
-                           3.0 * d.Py * d.Kx * 2 * nz * cplxb + (double)d.ncomp * Kz * Ky * d.Kx * realb);
+            LaunchScope ls(c, "fft_conv", zbytes);
             zconv_reg_kernel(d.Pz, 2 * nz <= d.Pz)<<<(unsigned)((cols + kZT - 1) / kZT), 3 * kZT, zconv_reg_smem(d.Pz),
                                                       c->stream>>>(z);
-        } else if (three_d && sizeof(T) == 4 && split_conv_supported(d.Pz)) {
-            split_conv_launch_3d(c, S, d.khat, nz, d.Py, d.Pz, d.Kx, d.Wk,
-                                 3.0 * d.Py * d.Kx * 2 * nz * cplxb + (double)d.ncomp * Kz * Ky * d.Kx * realb);
+        } else if (three_d ? launch_lane_z<T>(c, S, zbytes)
+                           : launch_lane_films<T>(c, d, S, ny, comp, 3 * comp, 1, "fft_conv", fbytes)) {
         } else if (three_d) {
             a.line_stride = plane; a.other_stride = d.Wk;
             a.L = d.Pz; a.n_in = nz; a.n_out = nz;
             a.tw = (const cplx<T>*)d.tw_z;
             a.kk_stride = Ky * d.Wk; a.ko_stride = d.Wk;
             a.L_other = d.Py; a.axis_is_y = 0;
-            launch_col<T, 0>(c, a, d.Py, "fft_conv",
-                             3.0 * d.Py * d.Kx * 2 * nz * cplxb + (double)d.ncomp * Kz * Ky * d.Kx * realb);
-        } else if (sizeof(T) == 4 && split_conv_supported(d.Py)) {
-            split_conv_launch_2d(c, S, d.khat, ny, d.Py, d.Kx, d.Wk, comp, 3 * comp, 1, "fft_conv",
-                                 3.0 * d.Kx * 2 * ny * cplxb + (double)d.ncomp * Ky * d.Kx * realb);
+            launch_col<T, 0>(c, a, d.Py, "fft_conv", zbytes);
         } else {
             a.line_stride = d.Wk; a.other_stride = plane;
             a.L = d.Py; a.n_in = ny; a.n_out = ny;
             a.tw = (const cplx<T>*)d.tw_y;
             a.kk_stride = d.Wk; a.ko_stride = 0;
             a.L_other = 1; a.axis_is_y = 1;
-            launch_col<T, 0>(c, a, 1, "fft_conv",
-                             3.0 * d.Kx * 2 * ny * cplxb + (double)d.ncomp * Ky * d.Kx * realb);
+            launch_col<T, 0>(c, a, 1, "fft_conv", fbytes);
         }
     }
-    if (three_d && d.Py > 1 && split_y) {
-        ysplit_launch(c, false, S, nz, d.Py, d.Kx, d.Wk, d.Py, ny, "fft_y_inv", 3.0 * nz * d.Kx * (ny + d.Py) * cplxb);
-    } else if (three_d && d.Py > 1 && fast_y) {
-        launch_y_direct(c, false, (cplx<float>*)S, plane, d.Py, ny, "fft_y_inv",
-                        3.0 * nz * d.Kx * (ny + d.Py) * cplxb);
-    } else if (three_d && d.Py > 1) {
+    if (three_d && d.Py > 1 && !launch_lane_y<T>(c, false, S, "fft_y_inv", ybytes)) {
         ColArgs<T> a{};
         a.base = S; a.comp_stride = comp; a.line_stride = d.Wk; a.other_stride = plane;
         a.nc = 3; a.Kx = d.Kx; a.L = d.Py; a.n_in = d.Py; a.n_out = ny;
         a.tw = (const cplx<T>*)d.tw_y;
-        launch_col<T, -1>(c, a, nz, "fft_y_inv", 3.0 * nz * d.Kx * (ny + d.Py) * cplxb);
+        launch_col<T, -1>(c, a, nz, "fft_y_inv", ybytes);
     }
     if (c2r)
         launch_x<T>(c, false, nullptr, Hd, S, 3 * nz * ny, ny, d.PyA, nx, nx, d.Lh, (const cplx<T>*)d.tw_x, false, N);
@@ -1346,10 +1361,8 @@ void demag_apply_stacked2d(mm_ctx* c, const DemagPlan& p, const float* m, float*
     const double cplxb = sizeof(cplx<float>), realb = sizeof(float);
     launch_x<float>(c, true, m, nullptr, Sp, 3 * ny * Rc, ny, p.PyA, nx, nx, p.Lh, (const cplx<float>*)p.tw_x, true,
                     N);
-    if (split_conv_supported(p.Py)) {
-        split_conv_launch_2d(c, Sp, p.khat, ny, p.Py, p.Kx, p.Wk, plane, 3 * plane, Rc, "fft_conv_stacked",
-                             Rc * (3.0 * p.Kx * 2 * ny * cplxb) + (double)p.ncomp * (p.Py / 2 + 1) * p.Kx * realb);
-    } else {
+    const double bytes = Rc * (3.0 * p.Kx * 2 * ny * cplxb) + (double)p.ncomp * (p.Py / 2 + 1) * p.Kx * realb;
+    if (!launch_lane_films<float>(c, p, Sp, ny, plane, 3 * plane, Rc, "fft_conv_stacked", bytes)) {
         ColArgs<float> a{};
         a.base = Sp; a.comp_stride = plane; a.nc = 3; a.Kx = p.Kx;
         a.khat = (const float*)p.khat;
@@ -1361,8 +1374,7 @@ void demag_apply_stacked2d(mm_ctx* c, const DemagPlan& p, const float* m, float*
         a.tw = (const cplx<float>*)p.tw_y;
         a.kk_stride = p.Wk; a.ko_stride = 0;
         a.L_other = 1; a.axis_is_y = 1;
-        launch_col<float, 0>(c, a, Rc, "fft_conv_stacked",
-                             Rc * (3.0 * p.Kx * 2 * ny * cplxb) + (double)p.ncomp * Ky * p.Kx * realb);
+        launch_col<float, 0>(c, a, Rc, "fft_conv_stacked", bytes);
     }
     launch_x<float>(c, false, nullptr, Hd, Sp, 3 * ny * Rc, ny, p.PyA, nx, nx, p.Lh, (const cplx<float>*)p.tw_x,
                     false, N);
@@ -1411,6 +1423,8 @@ static mm_status demag_setup_t(mm_ctx* c) {
     if (!make_plan(d.Lh, &tmp) || !make_plan(d.Py, &tmp) || !make_plan(d.Pz, &tmp))
         return set_error(c, MM_ERR_ARG, "internal: padded length is not 2^a 3^b");
 
+    if (const cudaError_t e = lane_attributes<T>(d, nz > 1); e != cudaSuccess)
+        return cuda_check(c, e, "column kernel attributes");
     // twiddles in working precision, and FP64 twiddles for the setup FFTs
     d.tw_x = make_twiddles<T>(d.Px);
     d.tw_y = make_twiddles<T>(d.Py);
@@ -1521,20 +1535,16 @@ static cudaError_t fft_attributes() {
         const int n = L == 0 ? 7 : L;
         if (e == cudaSuccess) e = smem_attr(x_kernel<T>(true, n));
         if (e == cudaSuccess) e = smem_attr(x_kernel<T>(false, n));
-        if (e == cudaSuccess) e = smem_attr(col_kernel<T, 1>(n));
-        if (e == cudaSuccess) e = smem_attr(col_kernel<T, -1>(n));
-        if (e == cudaSuccess) e = smem_attr(col_kernel<T, 0>(n));
     }
+    if (e == cudaSuccess) e = smem_attr(fft_col_kernel<T, 1>);
+    if (e == cudaSuccess) e = smem_attr(fft_col_kernel<T, -1>);
+    if (e == cudaSuccess) e = smem_attr(fft_col_kernel<T, 0>);
     return e;
 }
 
 static cudaError_t fast_attributes() {
     cudaError_t e = cudaSuccess;
-    for (int L : {16, 32, 48, 64, 81, 96, 108, 128, 162, 192, 216, 256, 324, 432, 512, 1024}) {
-        if (e == cudaSuccess) e = smem_attr(y_direct_kernel(true, L));
-        if (e == cudaSuccess) e = smem_attr(y_direct_kernel(false, L));
-    }
-    for (int L : {4, 8, 16, 32}) {
+    for (int L : {4, 8, 16}) {
         if (e == cudaSuccess) e = smem_attr(zconv_reg_kernel(L, false));
         if (e == cudaSuccess) e = smem_attr(zconv_reg_kernel(L, true));
     }
@@ -1557,7 +1567,6 @@ mm_status demag_setup(mm_ctx* c) {
         tw32[q] = make_float2((float)std::cos(ang), (float)std::sin(ang));
     }
     cudaError_t e = cudaMemcpyToSymbol(c_tw32, tw32, sizeof tw32);
-    if (e == cudaSuccess) e = split_conv_setup();
     if (e == cudaSuccess) e = field_c2r_setup();
     if (e != cudaSuccess) return cuda_check(c, e, "twiddle table");
     e = fft_attributes<float>();

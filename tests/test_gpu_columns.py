@@ -1,0 +1,86 @@
+"""GPU parity of the column passes at every line length that has a kernel of
+its own, and at both ends of the range of sizes that is padded to it: the
+middle pass of a film, of many films and of a 3-D grid, and the Y passes.
+The demag field is compared with the FP64 oracle's transforms; the bars are
+those of the field tests (an FP32 transform of these lengths rounds to a few
+1e-7 of the largest field, FP64 to a few 1e-16)."""
+import numpy as np
+import pytest
+
+import workloads as W
+from gpu_util import TERMS, make_ctx, need_gpu, oracle_problem, rel_err
+
+pytestmark = pytest.mark.gpu
+
+LENGTHS = sorted(2 ** a * 3 ** b for a in range(11) for b in range(7) if 2 <= 2 ** a * 3 ** b <= 1024)
+MAT = W.Material(Ms=8.0e5, A=1.3e-11, alpha=0.02)
+
+
+def _sizes(L):
+    """The smallest and the largest n that are padded to L (2n - 1 points)."""
+    below = max([v for v in LENGTHS if v < L], default=0)
+    return sorted({below // 2 + 1, (L + 1) // 2} - {1})
+
+
+def _check(grid, prec):
+    mm = need_gpu()
+    from oracle.demag import demag_spectrum, h_demag
+    ctx = make_ctx(mm, grid, MAT, precision=prec, demag=True)
+    try:
+        mm.mm_set_m(ctx, 0, W.m_random_sphere(grid, seed=grid.n))
+        m = mm.mm_get_m(ctx, 0, (3,) + grid.shape)
+        p = oracle_problem(grid, MAT)
+        ref = h_demag(m, p, demag_spectrum(p.shape, p.d))
+        H = mm.mm_get_heff(ctx, 0, m.shape, TERMS["demag"])
+        assert rel_err(H, ref) < (1e-11 if prec == 64 else 5e-6)
+    finally:
+        mm.mm_destroy(ctx)
+
+
+@pytest.mark.parametrize("prec", [64, 32])
+@pytest.mark.parametrize("L", [v for v in LENGTHS if v >= 12])
+def test_film_middle_pass(L, prec):
+    for ny in _sizes(L):
+        _check(W.Grid(5 if ny % 2 else 10, ny, 1, 2e-9, 2e-9, 1e-9), prec)
+
+
+@pytest.mark.parametrize("prec", [64, 32])
+@pytest.mark.parametrize("L", [v for v in LENGTHS if v >= 27])
+def test_y_passes(L, prec):
+    for ny in _sizes(L):
+        _check(W.Grid(3, ny, 2, 2e-9, 2e-9, 2e-9), prec)
+
+
+@pytest.mark.parametrize("prec", [64, 32])
+@pytest.mark.parametrize("L", [v for v in LENGTHS if 9 <= v <= 144])
+def test_z_middle_pass(L, prec):
+    for nz in _sizes(L):
+        _check(W.Grid(9, 6, nz, 3e-9, 3e-9, 3e-9), prec)
+
+
+@pytest.mark.parametrize("n", [16, 18, 27, 33, 54, 72, 81, 108])
+def test_many_films_match_one(n):
+    """Enough films for the kernel of ensembles: the first and the last
+    replica, two Heun steps, against the FP64 oracle."""
+    mm = need_gpu()
+    from oracle.llg import Solver
+    R = 2 * 160 * 32 // (n + 1) + 1
+    cell = (2e-9, 2e-9, 1e-9)
+    M = mm.Material(MAT.Ms, MAT.A, MAT.alpha)
+    cfg = mm.make_config(precision=32, integrator=mm.MM_HEUN, demag=mm.MM_DEMAG_EXACT, dt=1e-13)
+    ctx = mm.mm_create_batch([mm.make_grid(n, n, 1, *cell)] * R, M.s, cfg)
+    try:
+        mm.mm_batch_set_shape(ctx, 0)
+        g = W.Grid(n, n, 1, *cell)
+        m0 = {r: W.m_perp(g, seed=r, tilt=0.3) for r in (0, R - 1)}
+        for r, m in m0.items():
+            mm.mm_set_m(ctx, r, m)
+        mm.mm_step(ctx, 2)
+        p = oracle_problem(g, MAT)
+        for r, m in m0.items():
+            o = Solver(p, m, terms=("exchange", "zeeman", "demag"), dt=1e-13)
+            for _ in range(2):
+                o.heun_step()
+            assert np.abs(mm.mm_get_m(ctx, r, m.shape) - o.m).max() <= 1e-5
+    finally:
+        mm.mm_destroy(ctx)
