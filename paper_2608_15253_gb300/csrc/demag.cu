@@ -22,10 +22,10 @@
 #include "common.cuh"
 #include "ctx.h"
 #include "conv_lane.cuh"
-#include "fft_ct.cuh"
 #include "fft_direct.cuh"
 #include "fft_rt.cuh"
 #include "lane.h"
+#include "lane_x.cuh"
 
 namespace mm {
 
@@ -82,13 +82,14 @@ __device__ __forceinline__ long long spec_row(const XArgs<T>& a, int r) {
     return (long long)(r / a.rows_per_plane) * a.spec_rows_per_plane + (r % a.rows_per_plane);
 }
 
-// LT > 0: compile-time half length (specialised FFT), LT == 0: runtime plan
-template <typename T, int LT>
+// any half length 2^a 3^b (those without a lane kernel, and the full rows of
+// the tensor setup): runtime plan
+template <typename T>
 __global__ void __launch_bounds__(256) fft_x_r2c_kernel(XArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (a.stage > 0 && !a.st->active) return;
     cplx<T>* sm = reinterpret_cast<cplx<T>*>(smem_raw);
-    const int Lh = LT > 0 ? LT : a.Lh;
+    const int Lh = a.Lh;
     const int pitch = Lh + 1;
     const int r0 = blockIdx.x * a.rpc;
     const int nl = min(a.rpc, a.rows - r0);
@@ -116,8 +117,7 @@ __global__ void __launch_bounds__(256) fft_x_r2c_kernel(XArgs<T> a) {
     }
     __syncthreads();
     const int nin = (a.nx + 1) / 2;
-    if constexpr (LT > 0) ct_fft<T, 1, LT, LT + 1, 256, kMaxV>(sm, nl, nin, a.tw, 2);
-    else fft_lines<T, 1>(sm, nl, pitch, a.plan, nin, a.tw, 2);
+    fft_lines<T, 1>(sm, nl, pitch, a.plan, nin, a.tw, 2);
     // split: X[k] = (Z[k] + conj Z[M-k])/2 - i/2 W^k (Z[k] - conj Z[M-k])
     const int M = Lh, Kx = Lh + 1;
     for (int l = 0; l < nl; ++l) {
@@ -133,11 +133,11 @@ __global__ void __launch_bounds__(256) fft_x_r2c_kernel(XArgs<T> a) {
     }
 }
 
-template <typename T, int LT>
+template <typename T>
 __global__ void __launch_bounds__(256) fft_x_c2r_kernel(XArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* sm = reinterpret_cast<cplx<T>*>(smem_raw);
-    const int Lh = LT > 0 ? LT : a.Lh;
+    const int Lh = a.Lh;
     const int pitch = Lh + 1;
     const int r0 = blockIdx.x * a.rpc;
     const int nl = min(a.rpc, a.rows - r0);
@@ -166,359 +166,11 @@ __global__ void __launch_bounds__(256) fft_x_c2r_kernel(XArgs<T> a) {
         }
     }
     __syncthreads();
-    if constexpr (LT > 0) ct_fft<T, -1, LT, LT + 1, 256, kMaxV>(sm, nl, M, a.tw, 2);
-    else fft_lines<T, -1>(sm, nl, pitch, a.plan, M, a.tw, 2);
+    fft_lines<T, -1>(sm, nl, pitch, a.plan, M, a.tw, 2);
     const T* smr = reinterpret_cast<const T*>(sm);
     for (int l = 0; l < nl; ++l) {
         T* out = a.out_real + (long long)(r0 + l) * a.in_pitch;
         for (int q = threadIdx.x; q < a.nx; q += blockDim.x) out[q] = smr[2 * (l * pitch) + q];
-    }
-}
-
-// FP32 X passes with the first (R2C) or first and last (C2R) Stockham pass
-// working straight between global memory and registers.  Rows per CTA are a
-// compile-time constant (the same rule the host uses for the generic path).
-__host__ __device__ constexpr int x_rows_per_cta(int Lh) {
-    return (kMaxV * 256 / Lh) < 1 ? 1 : (kMaxV * 256 / Lh) > 16 ? 16 : (kMaxV * 256 / Lh);
-}
-
-template <int LT>
-__global__ void __launch_bounds__(256) fft_x_r2c_direct_kernel(XArgs<float> a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (a.stage > 0 && !a.st->active) return;
-    float2* sm = reinterpret_cast<float2*>(smem_raw);
-    constexpr int NT = 256, LP = LT + 1, RPC = x_rows_per_cta(LT);
-    constexpr int R0 = ct_radix(LT, 0), NB0 = LT / R0;
-    constexpr int MAXB = (RPC * NB0 + NT - 1) / NT;
-    const int r0 = blockIdx.x * a.rpc;            // a.rpc <= RPC (fewer rows per CTA on small grids)
-    const int nl = min(a.rpc, a.rows - r0);
-    const int nin = (a.nx + 1) / 2;
-    const int total = nl * NB0;
-    const bool vec2 = (a.nx % 2 == 0) && (a.in_pitch % 2 == 0);
-    // packed complex z[n] = Ms (x[2n] + i x[2n+1]), loaded into registers
-    float2 v[MAXB][R0];
-#pragma unroll
-    for (int i = 0; i < MAXB; ++i) {
-        const int b = threadIdx.x + i * NT;
-        if (b < total) {
-            const int l = b / NB0, j = b % NB0;
-            const long long g0 = (long long)(r0 + l) * a.in_pitch;
-#pragma unroll
-            for (int t = 0; t < R0; ++t) {
-                const int n = j + t * NB0;
-                float2 z = make_float2(0.f, 0.f);
-                if (n < nin) {
-                    const long long q = g0 + 2 * n;
-                    const bool has_y = 2 * n + 1 < a.nx;
-                    if (a.stage > 0) {
-                        // fused RK45 stage (nx even): form m_s, keep it, transform it
-                        const int kf = a.st->k_first;
-                        z.x = stage_value<float>(a, a.stage, kf, q);
-                        z.y = stage_value<float>(a, a.stage, kf, q + 1);
-                        *reinterpret_cast<float2*>(a.ms + q) = z;
-                    } else if (vec2) {
-                        z = *reinterpret_cast<const float2*>(a.in + q);
-                    } else {
-                        z.x = a.in[q];
-                        z.y = has_y ? a.in[q + 1] : 0.f;
-                    }
-                    if (a.region) {
-                        z.x *= a.lut[a.region[q % a.cells_per_comp]].Ms;
-                        z.y = has_y ? z.y * a.lut[a.region[(q + 1) % a.cells_per_comp]].Ms : 0.f;
-                    } else {
-                        z.x *= a.ms_uniform;
-                        z.y *= a.ms_uniform;
-                    }
-                }
-                v[i][t] = z;
-            }
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < MAXB; ++i) {
-        const int b = threadIdx.x + i * NT;
-        if (b < total) {
-            const int l = b / NB0, j = b % NB0;
-            dft_ct<float, 1, R0>(v[i]);
-#pragma unroll
-            for (int t = 0; t < R0; ++t) sm[l * LP + j * R0 + t] = v[i][t];
-        }
-    }
-    __syncthreads();
-    ct_fft<float, 1, LT, LP, NT, kMaxV, 1>(sm, nl, LT, a.tw, 2);
-    // split: X[k] = (Z[k] + conj Z[M-k])/2 - i/2 W^k (Z[k] - conj Z[M-k])
-    constexpr int M = LT, Kx = LT + 1;
-    for (int l = 0; l < nl; ++l) {
-        float2* out = a.spec + spec_row(a, r0 + l) * a.Wk;
-        for (int k = threadIdx.x; k < Kx; k += NT) {
-            const float2 zk = sm[l * LP + (k == M ? 0 : k)];
-            const float2 zc = cconj<float>(sm[l * LP + (k == 0 ? 0 : M - k)]);
-            const float2 E = cscale<float>(cadd<float>(zk, zc), 0.5f);
-            const float2 O = cscale<float>(mul_mi<float, 1>(csub<float>(zk, zc)), 0.5f);
-            const float2 w = __ldg(&a.tw[k]);
-            out[k] = cadd<float>(E, cmul<float>(w, O));
-        }
-    }
-}
-
-template <int LT>
-__global__ void __launch_bounds__(256) fft_x_c2r_direct_kernel(XArgs<float> a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2* sm = reinterpret_cast<float2*>(smem_raw);
-    constexpr int NT = 256, LP = LT + 1, RPC = x_rows_per_cta(LT), M = LT, Kx = LT + 1;
-    constexpr int NP = ct_npass(LT);
-    static_assert(NP >= 2, "first and last pass must differ");
-    const int r0 = blockIdx.x * a.rpc;            // a.rpc <= RPC (fewer rows per CTA on small grids)
-    const int nl = min(a.rpc, a.rows - r0);
-    for (int l = 0; l < nl; ++l) {
-        const float2* in = a.spec + spec_row(a, r0 + l) * a.Wk;
-        for (int k = threadIdx.x; k < Kx; k += NT) sm[l * LP + k] = in[k];
-    }
-    __syncthreads();
-    // first pass, fed by the rebuild Z'[k] = (X[k] + conj X[M-k]) + i (X[k] - conj X[M-k]) conj(W^k)
-    {
-        constexpr int R0 = ct_radix(LT, 0), NB0 = LT / R0;
-        constexpr int MAXB = (RPC * NB0 + NT - 1) / NT;
-        const int total = nl * NB0;
-        float2 v[MAXB][R0];
-#pragma unroll
-        for (int i = 0; i < MAXB; ++i) {
-            const int b = threadIdx.x + i * NT;
-            if (b < total) {
-                const int l = b / NB0, j = b % NB0;
-#pragma unroll
-                for (int t = 0; t < R0; ++t) {
-                    const int k = j + t * NB0;
-                    const float2 xk = sm[l * LP + k];
-                    const float2 xc = cconj<float>(sm[l * LP + M - k]);
-                    const float2 w = __ldg(&a.tw[k]);
-                    const float2 E = cadd<float>(xk, xc);
-                    const float2 O = cmulc<float>(csub<float>(xk, xc), w);
-                    v[i][t] = cadd<float>(E, mul_mi<float, -1>(O));
-                }
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < MAXB; ++i) {
-            const int b = threadIdx.x + i * NT;
-            if (b < total) {
-                const int l = b / NB0, j = b % NB0;
-                dft_ct<float, -1, R0>(v[i]);
-#pragma unroll
-                for (int t = 0; t < R0; ++t) sm[l * LP + j * R0 + t] = v[i][t];
-            }
-        }
-        __syncthreads();
-    }
-    ct_fft<float, -1, LT, LP, NT, kMaxV, 1, NP - 1>(sm, nl, LT, a.tw, 2);
-    // last pass straight to the real rows: z[n] -> (x[2n], x[2n+1])
-    {
-        constexpr int P = NP - 1, R = ct_radix(LT, P), NS = ct_ns(LT, P), NB = LT / R;
-        static_assert(NB == NS, "last pass writes natural order");
-        constexpr int MAXB = (RPC * NB + NT - 1) / NT;
-        const int total = nl * NB;
-        const bool vec2 = (a.nx % 2 == 0) && (a.in_pitch % 2 == 0);
-#pragma unroll
-        for (int i = 0; i < MAXB; ++i) {
-            const int b = threadIdx.x + i * NT;
-            if (b < total) {
-                const int l = b / NB, j = b % NB;
-                float2 v[R];
-#pragma unroll
-                for (int t = 0; t < R; ++t) v[t] = sm[l * LP + j + t * NB];
-#pragma unroll
-                for (int t = 1; t < R; ++t) v[t] = cmulc<float>(v[t], __ldg(&a.tw[(t * j) * 2]));
-                dft_ct<float, -1, R>(v);
-                float* out = a.out_real + (long long)(r0 + l) * a.in_pitch;
-#pragma unroll
-                for (int t = 0; t < R; ++t) {
-                    const int n = j + t * NS;
-                    if (2 * n + 1 < a.nx) {
-                        if (vec2) *reinterpret_cast<float2*>(out + 2 * n) = v[t];
-                        else { out[2 * n] = v[t].x; out[2 * n + 1] = v[t].y; }
-                    } else if (2 * n < a.nx) {
-                        out[2 * n] = v[t].x;
-                    }
-                }
-            }
-        }
-    }
-}
-
-// FP32 X passes for rows of half length 64 ... 512: one row per warp, eight
-// warps per CTA, no CTA-wide barrier.  R2C: packed pairs straight from global memory
-// into the first pass, later passes in warp-private shared memory, then the
-// split to the Lh+1 spectrum.  C2R: the rebuild of Z' from X[k] and
-// X[M-k] (both read from global memory) feeds the first pass; the last pass
-// writes the real row.
-constexpr int kXW = 8;   // warps (rows) per CTA
-
-// Slot of stage j's slope under the first-same-as-last rotation (slots 0
-// and 6 swap roles between steps).
-__device__ __forceinline__ int stage_slot(int j, int k_first) {
-    return j == 0 ? k_first : j == 6 ? 6 - k_first : j;
-}
-
-// m_s = m0 + sum_{j<S} (dt a_sj) k_j at the float2 pair starting at q
-template <int S>
-__device__ __forceinline__ float2 stage_pair(const XArgs<float>& a, const float* cf, int kf, long long q) {
-    float2 acc = __ldg(reinterpret_cast<const float2*>(a.m0 + q));
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-        if (j == 1 && S == 6) continue;             // a_7,2 = 0
-        const float2 k = __ldg(reinterpret_cast<const float2*>(a.kptr[stage_slot(j, kf)] + q));
-        acc.x += cf[j] * k.x;
-        acc.y += cf[j] * k.y;
-    }
-    return acc;
-}
-
-// S = 0: rows of a.in.  S >= 1 (RK45 stage S, nx even): rows of the stage
-// state formed from m0 and the slopes, which is also stored to a.ms; the
-// whole launch is a no-op when the attempt is inactive.
-// (at most 64 registers: four CTAs of 8 warps per SM; 512x512x64 stage
-// transform 412 -> 385 us against the unconstrained 80)
-template <int LT, int S>
-__global__ void __launch_bounds__(32 * kXW, 4) fft_x_r2c_warp_kernel(XArgs<float> a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (S > 0 && !a.st->active) return;
-    // a group of GW lanes per row (a warp takes 32 / GW rows of a short line)
-    constexpr int GW = warp_group(LT), RPW = 32 / GW;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & (GW - 1);
-    const int wrow = (blockIdx.x * kXW + warp) * RPW;
-    if (wrow >= a.rows) return;                 // whole warp: no CTA barrier below
-    const int slot = warp * RPW + (threadIdx.x & 31) / GW;
-    const bool rvalid = wrow + (threadIdx.x & 31) / GW < a.rows;
-    const int row = rvalid ? wrow + (threadIdx.x & 31) / GW : wrow;   // a spare group repeats the first row
-    float2* sm = reinterpret_cast<float2*>(smem_raw) + slot * wline(LT);
-    constexpr int NP = ct_npass(LT);
-    const int nin = (a.nx + 1) / 2;
-    const long long g0 = (long long)row * a.in_pitch;
-    const bool vec2 = (a.nx % 2 == 0) && (a.in_pitch % 2 == 0);
-    const float* cf = S > 0 ? a.st->cf32[S] : nullptr;
-    const int kf = S > 0 ? a.st->k_first : 0;
-    auto load_in = [&](int n) {
-        float2 z = make_float2(0.f, 0.f);
-        if (n < nin) {
-            const long long q = g0 + 2 * n;
-            const bool has_y = 2 * n + 1 < a.nx;
-            if constexpr (S > 0) {
-                z = stage_pair<S>(a, cf, kf, q);
-                if (rvalid) *reinterpret_cast<float2*>(a.ms + q) = z;
-            } else if (vec2) {
-                z = *reinterpret_cast<const float2*>(a.in + q);
-            } else {
-                z.x = a.in[q];
-                z.y = has_y ? a.in[q + 1] : 0.f;
-            }
-            if (a.region) {
-                z.x *= a.lut[a.region[q % a.cells_per_comp]].Ms;
-                z.y = has_y ? z.y * a.lut[a.region[(q + 1) % a.cells_per_comp]].Ms : 0.f;
-            } else {
-                z.x *= a.ms_uniform;
-                z.y *= a.ms_uniform;
-            }
-        }
-        return z;
-    };
-    warp_pass<float, 1, LT, ct_radix(LT, 0), 1, GW>(a.tw, 2, load_in, [&](int i, float2 v) { sm[wpad(i)] = v; });
-    warp_fft_smem<float, 1, LT, 1, NP, GW>(sm, a.tw, 2);
-    constexpr int M = LT, Kx = LT + 1;
-    float2* out = a.spec + spec_row(a, row) * a.Wk;
-    for (int k = lane; k < Kx; k += GW) {
-        const float2 zk = sm[wpad(k == M ? 0 : k)];
-        const float2 zc = cconj<float>(sm[wpad(k == 0 ? 0 : M - k)]);
-        const float2 E = cscale<float>(cadd<float>(zk, zc), 0.5f);
-        const float2 O = cscale<float>(mul_mi<float, 1>(csub<float>(zk, zc)), 0.5f);
-        if (rvalid) out[k] = cadd<float>(E, cmul<float>(__ldg(&a.tw[k]), O));
-    }
-}
-
-template <int LT>
-__global__ void __launch_bounds__(32 * kXW) fft_x_c2r_warp_kernel(XArgs<float> a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int GW = warp_group(LT), RPW = 32 / GW;
-    const int warp = threadIdx.x >> 5;
-    const int wrow = (blockIdx.x * kXW + warp) * RPW;
-    if (wrow >= a.rows) return;                 // whole warp
-    const int slot = warp * RPW + (threadIdx.x & 31) / GW;
-    const bool rvalid = wrow + (threadIdx.x & 31) / GW < a.rows;
-    const int row = rvalid ? wrow + (threadIdx.x & 31) / GW : wrow;   // a spare group repeats the first row
-    float2* sm = reinterpret_cast<float2*>(smem_raw) + slot * wline(LT);
-    float* out = a.out_real + (long long)row * a.in_pitch;
-    const bool vec2 = (a.nx % 2 == 0) && (a.in_pitch % 2 == 0);
-    const int nx = a.nx;
-    warp_c2r<LT, GW>(a.spec + spec_row(a, row) * a.Wk, a.tw, sm, [&](int n, float2 v) {
-        if (!rvalid) return;
-        if (2 * n + 1 < nx) {
-            if (vec2) *reinterpret_cast<float2*>(out + 2 * n) = v;
-            else { out[2 * n] = v.x; out[2 * n + 1] = v.y; }
-        } else if (2 * n < nx) {
-            out[2 * n] = v.x;
-        }
-    });
-}
-
-// C2R with the spectrum rows prefetched: persistent warps, each with two
-// line buffers in shared memory.  While a warp transforms one row (in place
-// in one buffer), cp.async brings its next row into the other, so the
-// global-memory latency of a row hides behind the transform of the previous
-// one instead of stalling the first pass.
-__device__ __forceinline__ void cpa16(void* smem, const void* gmem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cpa8(void* smem, const void* gmem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cpa_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
-// float2 per line buffer: the padded line, rounded to 16 bytes
-template <int LT> constexpr int xpipe_buf() { return (wline(LT) + 1) & ~1; }
-template <int LT> constexpr size_t xpipe_smem() { return (size_t)kXW * 2 * xpipe_buf<LT>() * sizeof(float2); }
-
-template <int LT>
-__global__ void __launch_bounds__(32 * kXW, 3) fft_x_c2r_pipe_kernel(XArgs<float> a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int BS = xpipe_buf<LT>();
-    static_assert(LT % 2 == 0, "16-byte pieces of the half spectrum");
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float2* buf = reinterpret_cast<float2*>(smem_raw) + warp * 2 * BS;
-    const int nw = gridDim.x * kXW;
-    float* const out0 = a.out_real;
-    const bool vec2 = (a.nx % 2 == 0) && (a.in_pitch % 2 == 0);
-    const int nx = a.nx;
-    // row r's LT + 1 spectrum values (16-byte aligned: the pitch Wk is even)
-    auto fetch = [&](int r, float2* dst) {
-        const float2* src = a.spec + spec_row(a, r) * a.Wk;
-        for (int q = lane; q < LT / 2; q += 32) cpa16(dst + 2 * q, src + 2 * q);
-        if (lane == 0) cpa8(dst + LT, src + LT);
-        cpa_commit();
-    };
-    int row = blockIdx.x * kXW + warp;
-    if (row < a.rows) fetch(row, buf);
-    for (int it = 0; row < a.rows; ++it, row += nw) {
-        float2* cur = buf + (it & 1) * BS;
-        if (row + nw < a.rows) {
-            fetch(row + nw, buf + ((it + 1) & 1) * BS);
-            cpa_wait<1>();
-        } else {
-            cpa_wait<0>();
-        }
-        __syncwarp();
-        float* out = out0 + (long long)row * a.in_pitch;
-        warp_c2r_inplace<LT>(cur, a.tw, [&](int n, float2 v) {
-            if (2 * n + 1 < nx) {
-                if (vec2) *reinterpret_cast<float2*>(out + 2 * n) = v;
-                else { out[2 * n] = v.x; out[2 * n + 1] = v.y; }
-            } else if (2 * n < nx) {
-                out[2 * n] = v.x;
-            }
-        });
     }
 }
 
@@ -978,83 +630,6 @@ static int col_tk(int L, int nc) {
     return tk;
 }
 
-// Lengths with a compile-time FFT (FP32): every half-length and column
-// length of the benchmark workloads; other lengths and FP64 take the
-// runtime-planned path.
-#define MM_CT_LENGTHS(X) \
-    X(16) X(32) X(48) X(64) X(81) X(96) X(108) X(128) X(162) X(192) X(216) X(256) X(324) X(432) X(512) X(1024)
-
-template <typename T> using XKern = void (*)(XArgs<T>);
-
-template <typename T>
-static XKern<T> x_kernel(bool fwd, int Lh) {
-    if constexpr (sizeof(T) == 4) {
-        switch (Lh) {
-#define MM_CASE(n) case n: return fwd ? fft_x_r2c_direct_kernel<n> : fft_x_c2r_direct_kernel<n>;
-            MM_CT_LENGTHS(MM_CASE)
-#undef MM_CASE
-            default: break;
-        }
-    }
-    return fwd ? fft_x_r2c_kernel<T, 0> : fft_x_c2r_kernel<T, 0>;
-}
-
-// lanes per row of the one-row-per-warp kernels (warp_group of the length)
-static int x_warp_group(int Lh) {
-    switch (Lh) {
-#define MM_CASE(n) case n: return warp_group(n);
-        MM_CASE(32) MM_CASE(48) MM_CASE(64) MM_CASE(96) MM_CASE(128) MM_CASE(192) MM_CASE(216) MM_CASE(256) MM_CASE(324) MM_CASE(432)
-        MM_CASE(512)
-#undef MM_CASE
-        default: return 32;
-    }
-}
-
-static XKern<float> x_warp_kernel(bool fwd, int Lh) {
-    switch (Lh) {
-#define MM_CASE(n) case n: return fwd ? fft_x_r2c_warp_kernel<n, 0> : fft_x_c2r_warp_kernel<n>;
-        MM_CASE(32) MM_CASE(48) MM_CASE(64) MM_CASE(96) MM_CASE(128) MM_CASE(192) MM_CASE(216) MM_CASE(256) MM_CASE(324) MM_CASE(432)
-        MM_CASE(512)
-#undef MM_CASE
-        default: return nullptr;
-    }
-}
-
-// prefetching C2R (persistent warps); null where the plain warp kernel is used
-#define MM_XPIPE_LENGTHS(X) X(256) X(512)
-static XKern<float> x_c2r_pipe_kernel(int Lh) {
-    switch (Lh) {
-#define MM_CASE(n) case n: return fft_x_c2r_pipe_kernel<n>;
-        MM_XPIPE_LENGTHS(MM_CASE)
-#undef MM_CASE
-        default: return nullptr;
-    }
-}
-static size_t x_c2r_pipe_smem(int Lh) {
-    switch (Lh) {
-#define MM_CASE(n) case n: return xpipe_smem<n>();
-        MM_XPIPE_LENGTHS(MM_CASE)
-#undef MM_CASE
-        default: return 0;
-    }
-}
-
-// R2C fused with RK45 stage s (1..6); null where the warp path does not apply
-static XKern<float> x_stage_kernel(int s, int Lh) {
-#define MM_ST(n) \
-    case n: { \
-        static XKern<float> const t[7] = {nullptr, fft_x_r2c_warp_kernel<n, 1>, fft_x_r2c_warp_kernel<n, 2>, \
-                                          fft_x_r2c_warp_kernel<n, 3>, fft_x_r2c_warp_kernel<n, 4>, \
-                                          fft_x_r2c_warp_kernel<n, 5>, fft_x_r2c_warp_kernel<n, 6>}; \
-        return (s >= 1 && s <= 6) ? t[s] : nullptr; \
-    }
-    switch (Lh) {
-        MM_ST(192) MM_ST(216) MM_ST(256) MM_ST(324) MM_ST(432) MM_ST(512)
-        default: return nullptr;
-    }
-#undef MM_ST
-}
-
 using ZKern = void (*)(ZArgs<float>);
 
 // half: nz <= Pz/2 (the zero-padded upper half of every z line is known)
@@ -1103,41 +678,34 @@ static void launch_x(mm_ctx* c, bool forward, const T* in, T* out_real, cplx<T>*
     }
     a.cells_per_comp = cells_per_comp;
     a.stage = stage;
-    if constexpr (sizeof(T) == 4) {
-        if (stage > 0 && x_stage_kernel(stage, Lh)) {
-            // stage s reads m0 and the s slopes (s - 1 at stage 7), writes m_s and the spectrum
-            const double reads = (double)(1 + stage - (stage == 6 ? 1 : 0));
-            const size_t smem = (size_t)kXW * wline(Lh) * sizeof(float2);
-            LaunchScope ls(c, "fft_x_r2c_stage",
-                           (double)rows * ((reads + 1.0) * nx * sizeof(T) + (Lh + 1) * sizeof(cplx<T>)));
-            x_stage_kernel(stage, Lh)<<<(rows + kXW - 1) / kXW, 32 * kXW, smem, c->stream>>>(a);
+    const double reads = stage > 0 ? (double)(1 + stage - (stage == 6 ? 1 : 0)) + 1.0 : 1.0;
+    const char* name = stage > 0 ? "fft_x_r2c_stage" : forward ? "fft_x_r2c" : "fft_x_c2r";
+    const double bytes = (double)rows * (reads * nx * sizeof(T) + (Lh + 1) * sizeof(cplx<T>));
+    const XLane<T> xl = lane_x<T>(Lh);
+    if (xl.r2c && nx <= Lh) {                    // (the tensor setup transforms full rows)
+        XLaneArgs<T> x{};
+        x.in = in; x.out = out_real; x.spec = spec;
+        x.rows = rows; x.rows_per_plane = rows_per_plane; x.spec_rows_per_plane = spec_rows_per_plane;
+        x.nx = nx; x.Wk = a.Wk; x.cells = cells_per_comp; x.tw = tw;
+        x.ms = a.ms_uniform; x.region = a.region; x.lut = a.lut;
+        x.st = a.st; x.m0 = a.m0; x.ms_out = a.ms; x.stage = stage;
+        for (int q = 0; q < 7; ++q) x.k[q] = (const T*)c->d_k[q];
+        if (xl.fine_r2c && rows < 10 * sm_count()) {
+            // FP64 rows too few to fill the schedulers with the lanes' long
+            // instruction streams: a row per warp, one warp per CTA to reach
+            // every SM (R2C of 96 or 400 rows of 128: 8.3 against 18.5 us; 3072
+            // rows of 64: 24.6 against 18.5)
+            LaunchScope ls(c, name, bytes);
+            (forward ? xl.fine_r2c : xl.fine_c2r)<<<rows, 32, xl.fine_line, c->stream>>>(x);
             return;
         }
-        if (!forward && stage == 0 && x_c2r_pipe_kernel(Lh) && c->dm.Wk % 2 == 0) {
-            static int occ_by_len[2] = {0, 0};     // Lh = 256, 512
-            int& occ = occ_by_len[Lh == 512 ? 1 : 0];
-            if (!occ) {
-                int o = 0;
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, x_c2r_pipe_kernel(Lh), 32 * kXW,
-                                                              x_c2r_pipe_smem(Lh));
-                occ = std::max(1, o);
-            }
-            const int grid = std::max(1, std::min((rows + kXW - 1) / kXW, occ * sm_count()));
-            LaunchScope ls(c, "fft_x_c2r", (double)rows * (nx * sizeof(T) + (Lh + 1) * sizeof(cplx<T>)));
-            x_c2r_pipe_kernel(Lh)<<<grid, 32 * kXW, x_c2r_pipe_smem(Lh), c->stream>>>(a);
-            return;
-        }
-        // the plain one-row-per-warp kernels take no stage combine: with a
-        // stage to form they are only used through x_stage_kernel above
-        XKern<float> wk = stage == 0 ? x_warp_kernel(forward, Lh) : nullptr;
-        if (wk) {
-            const int rpc = kXW * (32 / x_warp_group(Lh));      // rows per CTA
-            const size_t smem = (size_t)rpc * wline(Lh) * sizeof(float2);
-            LaunchScope ls(c, forward ? "fft_x_r2c" : "fft_x_c2r",
-                           (double)rows * (nx * sizeof(T) + (Lh + 1) * sizeof(cplx<T>)));
-            wk<<<(rows + rpc - 1) / rpc, 32 * kXW, smem, c->stream>>>(a);
-            return;
-        }
+        // small grids: fewer rows per CTA so that two CTAs per SM run, whole warps where rows share one
+        const int unit = 32 % xl.group == 0 ? 32 / xl.group : 1;
+        int rpc = std::max(1, (rows + 2 * sm_count() - 1) / (2 * sm_count()));
+        rpc = std::min(xl.rows, (rpc + unit - 1) / unit * unit);
+        LaunchScope ls(c, name, bytes);
+        (forward ? xl.r2c : xl.c2r)<<<(rows + rpc - 1) / rpc, rpc * xl.group, rpc * xl.line, c->stream>>>(x);
+        return;
     }
     int rpc = std::max(1, kMaxV * 256 / Lh);
     rpc = std::min(rpc, 16);
@@ -1146,10 +714,8 @@ static void launch_x(mm_ctx* c, bool forward, const T* in, T* out_real, cplx<T>*
     rpc = std::max(1, std::min(rpc, (rows + 2 * sm_count() - 1) / (2 * sm_count())));
     a.rpc = rpc;
     const int grid = (rows + rpc - 1) / rpc;
-    const double reads = stage > 0 ? (double)(1 + stage - (stage == 6 ? 1 : 0)) + 1.0 : 1.0;
-    LaunchScope ls(c, stage > 0 ? "fft_x_r2c_stage" : forward ? "fft_x_r2c" : "fft_x_c2r",
-                   (double)rows * (reads * nx * sizeof(T) + (Lh + 1) * sizeof(cplx<T>)));
-    x_kernel<T>(forward, Lh)<<<grid, 256, smem, c->stream>>>(a);
+    LaunchScope ls(c, name, bytes);
+    (forward ? fft_x_r2c_kernel<T> : fft_x_c2r_kernel<T>)<<<grid, 256, smem, c->stream>>>(a);
 }
 
 template <typename T, int MODE>
@@ -1269,7 +835,10 @@ static cudaError_t lane_attributes(const DemagPlan& d, bool three_d) {
             const cudaError_t e = cudaFuncSetAttribute(k.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
             if (e != cudaSuccess) return e;
         }
-    return cudaSuccess;
+    const XLane<T> x = lane_x<T>(d.Lh);
+    if (!x.r2c) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(x.r2c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(x.rows * x.line));
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(x.c2r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(x.rows * x.line));
 }
 
 // c2r = false: every pass but the inverse X pass (which the fused inverse-X +
@@ -1386,17 +955,19 @@ void demag_apply(mm_ctx* c, const void* m, void* Hd) {
     else demag_apply_t<double>(c, (const double*)m, (double*)Hd);
 }
 
-// The one-row-per-warp X pass takes the stage combine at no cost; the
-// CTA-wide R2C kernels read the slopes with scalar loads, which only pays
-// on small grids where launches, not bandwidth, set the time (measured:
-// 10 K cells faster, 540 K cells 10 % slower fused).
+// The lane X kernels take the stage combine at no cost; the runtime-planned
+// one reads the slopes with scalar loads, which only pays on small grids where
+// launches, not bandwidth, set the time (measured: 10 K cells faster, 540 K
+// cells 10 % slower fused).
 bool demag_stage_fusable(const mm_ctx* c) {
-    if (c->prec != 32 || !c->dm.on || c->grid.nx % 2 != 0) return false;
-    return x_stage_kernel(1, c->dm.Lh) != nullptr || c->N <= 131072;
+    if (!c->dm.on) return false;
+    if (c->prec == 64) return lane_x<double>(c->dm.Lh).r2c != nullptr;
+    return lane_x<float>(c->dm.Lh).r2c != nullptr || c->N <= 131072;
 }
 
 void demag_apply_stage(mm_ctx* c, int stage, void* Hd) {
-    demag_apply_t<float>(c, (const float*)c->d_mtmp, (float*)Hd, stage);
+    if (c->prec == 32) demag_apply_t<float>(c, (const float*)c->d_mtmp, (float*)Hd, stage);
+    else demag_apply_t<double>(c, (const double*)c->d_mtmp, (double*)Hd, stage);
 }
 
 void demag_apply_partial(mm_ctx* c, const void* m, int stage) {
@@ -1528,33 +1099,14 @@ static cudaError_t smem_attr(K k) {
 
 template <typename T>
 static cudaError_t fft_attributes() {
-    static const int lengths[] = {0, 16, 32, 48, 64, 81, 96, 108, 128, 162, 192, 216, 256, 324, 432, 512, 1024};
-    cudaError_t e = cudaSuccess;
-    for (int L : lengths) {
-        if (L != 0 && sizeof(T) != 4) continue;
-        const int n = L == 0 ? 7 : L;
-        if (e == cudaSuccess) e = smem_attr(x_kernel<T>(true, n));
-        if (e == cudaSuccess) e = smem_attr(x_kernel<T>(false, n));
-    }
+    cudaError_t e = smem_attr(fft_x_r2c_kernel<T>);
+    if (e == cudaSuccess) e = smem_attr(fft_x_c2r_kernel<T>);
     if (e == cudaSuccess) e = smem_attr(fft_col_kernel<T, 1>);
     if (e == cudaSuccess) e = smem_attr(fft_col_kernel<T, -1>);
     if (e == cudaSuccess) e = smem_attr(fft_col_kernel<T, 0>);
-    return e;
-}
-
-static cudaError_t fast_attributes() {
-    cudaError_t e = cudaSuccess;
     for (int L : {4, 8, 16}) {
-        if (e == cudaSuccess) e = smem_attr(zconv_reg_kernel(L, false));
-        if (e == cudaSuccess) e = smem_attr(zconv_reg_kernel(L, true));
-    }
-    for (int L : {256, 512})
-        if (e == cudaSuccess) e = smem_attr(x_c2r_pipe_kernel(L));
-    for (int L : {192, 216, 256, 324, 432, 512}) {
-        if (e == cudaSuccess) e = smem_attr(x_warp_kernel(true, L));
-        if (e == cudaSuccess) e = smem_attr(x_warp_kernel(false, L));
-        for (int st = 1; st <= 6; ++st)
-            if (e == cudaSuccess) e = smem_attr(x_stage_kernel(st, L));
+        if (e == cudaSuccess && sizeof(T) == 4) e = smem_attr(zconv_reg_kernel(L, false));
+        if (e == cudaSuccess && sizeof(T) == 4) e = smem_attr(zconv_reg_kernel(L, true));
     }
     return e;
 }
@@ -1570,7 +1122,6 @@ mm_status demag_setup(mm_ctx* c) {
     if (e == cudaSuccess) e = field_c2r_setup();
     if (e != cudaSuccess) return cuda_check(c, e, "twiddle table");
     e = fft_attributes<float>();
-    if (e == cudaSuccess) e = fast_attributes();
     if (e == cudaSuccess) e = fft_attributes<double>();
     if (e != cudaSuccess) return cuda_check(c, e, "FFT kernel attributes");
     return c->prec == 32 ? demag_setup_t<float>(c) : demag_setup_t<double>(c);

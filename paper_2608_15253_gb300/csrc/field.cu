@@ -15,7 +15,7 @@
 #include "common.cuh"
 #include "ctx.h"
 #include "field_dev.cuh"
-#include "fft_direct.cuh"
+#include "lane_x.cuh"
 
 namespace mm {
 
@@ -260,53 +260,50 @@ __global__ void __launch_bounds__(256) field_vec_kernel(FieldArgs<float> a) {
 }
 
 // The last demag pass (inverse X, half spectrum -> real rows) fused with
-// the field kernel: a CTA of kC2RWarps = 4 warps takes kC2RRows = 4 rows
-// (z, y); its warps transform the three components of those rows (one row
-// of one component per warp at a time, three each) into shared memory, then
-// every thread forms the field, torque and stage output of 4 cells at a time
-// with the demag field read from there -- H_demag never goes through global
-// memory.
+// the field kernel: the first 3 G rows_per_cta threads of a CTA run the C2R of
+// the three components of its rows (z, y), G threads each (lane_x.cuh), into
+// shared memory over the exchange buffers; then every thread forms the field,
+// torque and stage output of 4 cells at a time with the demag field read from
+// there -- H_demag never goes through global memory.
 struct C2RSpec {
     const float2* spec;     // [3][nz][PyA][Wk]
     const float2* tw;       // exp(-2 pi i q / Px)
     int PyA, Wk;
+    int rpc;                // rows per CTA
 };
 
-constexpr int kC2RRows = 4;
-constexpr int kC2RWarps = 4;
-constexpr int kC2RThreads = 32 * kC2RWarps;
-template <int LT>
-constexpr size_t c2r_field_smem() {
-    return (size_t)kC2RWarps * wline(LT) * sizeof(float2) + (size_t)3 * kC2RRows * LT * sizeof(float);
+constexpr int kC2RThreads = 192;
+// exchange lines of the C2R threads in whole warps, and the field rows over them
+template <int M, int G, int Q>
+constexpr size_t c2r_field_smem(int rpc) {
+    const size_t tasks = (3 * rpc * G + 31) / 32 * 32 / G;
+    const size_t lines = tasks * XSplit<M, G, Q>::LINE * sizeof(float2), rows = (size_t)3 * rpc * M * sizeof(float);
+    return lines > rows ? lines : rows;
 }
 
-// Four 4-warp CTAs per SM for the QUIET form (128 registers, no spills):
-// as many warps as two CTAs of 8, but more CTAs at different phases -- 4 %
-// faster on rows of 512.  The full form is left uncapped (156-218
-// registers, two or three CTAs per SM) rather than spill.
-template <int LT, bool EXT, bool QUIET = false>
-__global__ void __launch_bounds__(kC2RThreads, QUIET ? 4 : 1) c2r_field_kernel(FieldArgs<float> a, C2RSpec s) {
+template <int M, int G, int Q, bool EXT, bool QUIET = false>
+__global__ void __launch_bounds__(kC2RThreads, QUIET ? 2 : 1) c2r_field_kernel(FieldArgs<float> a, C2RSpec s) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (a.gate && !a.st->active) return;
-    const int warp = threadIdx.x >> 5;
-    float2* line = reinterpret_cast<float2*>(smem_raw) + warp * wline(LT);
-    float* sH = reinterpret_cast<float*>(smem_raw + (size_t)kC2RWarps * wline(LT) * sizeof(float2));   // [rpc][3][nx]
-    const int nx = a.nx, rpc = kC2RRows, nrows = a.ny * a.nz;
+    float* sH = reinterpret_cast<float*>(smem_raw);   // [rpc][3][nx], once the lines are in registers
+    const int nx = a.nx, rpc = s.rpc, nrows = a.ny * a.nz;
     const int row0 = blockIdx.x * rpc;
-    for (int task = warp; task < 3 * rpc; task += kC2RWarps) {
-        const int rl = task / 3, comp = task - 3 * rl, row = row0 + rl;
-        if (row >= nrows) break;                      // warp-uniform; later tasks have larger rows
-        const int z = row / a.ny, y = row - z * a.ny;
+    if ((int)threadIdx.x < (3 * rpc * G + 31) / 32 * 32) {
+        const int task = threadIdx.x / G, rl = task / 3, comp = task - 3 * rl, row = row0 + rl;
+        const bool valid = rl < rpc && row < nrows;
+        const int z = valid ? row / a.ny : 0, y = valid ? row - z * a.ny : 0;
         const float2* X = s.spec + ((long long)(comp * a.nz + z) * s.PyA + y) * s.Wk;
+        lcx<float>* line = reinterpret_cast<lcx<float>*>(smem_raw) + task * XSplit<M, G, Q>::LINE;
         float* dst = sH + (rl * 3 + comp) * nx;
-        warp_c2r<LT>(X, s.tw, line, [&](int n, float2 v) {
-            if (2 * n + 1 < nx) *reinterpret_cast<float2*>(dst + 2 * n) = v;
+        lane_c2r_row<float, M, G, Q>(X, s.tw, line, threadIdx.x % G, valid, [] { __syncthreads(); }, [&](int n, float2 v) {
+            if (valid && 2 * n < nx) *reinterpret_cast<float2*>(dst + 2 * n) = v;
         });
-        __syncwarp();
+    } else {
+        __syncthreads();
     }
     __syncthreads();
     const int tpr = nx / 4;
-    for (int c = threadIdx.x; c < rpc * tpr; c += kC2RThreads) {
+    for (int c = threadIdx.x; c < rpc * tpr; c += blockDim.x) {
         const int rl = c / tpr, x0 = 4 * (c - rl * tpr);
         const int row = row0 + rl;
         if (row < nrows) {
@@ -439,37 +436,44 @@ void field_launch(mm_ctx* c, int mode, unsigned terms, const void* m, const void
 }
 
 // Inverse X pass + field kernel in one launch (FP32, one material, nx a
-// multiple of 4 dividing 1024, the one-row-per-warp inverse X transform of
-// the grid's half length available).  Measured against the two separate
-// kernels: 37.6 against 18.2 + 22.4 us per 256x256x16 evaluation; at
-// nx = 512 with the QUIET field variant 385 against 198 + 201 us (the
-// general field variant had made it slower there: 430 against 204 + 215).
-#define MM_C2R_FIELD_LENGTHS(X) X(128) X(256) X(512)
+// multiple of 4 dividing 1024 and equal to the half length).  One GB300:
+// 512x512x64 293 us (307 with a row per warp and three transforms in turn),
+// 256x256x16 26.6 (27.9), a 512x512 film 12.8 (16.7), a 256x256 film at 300 K
+// with spin-orbit torque 14.8 (19.9).  The two separate kernels take 198 + 201
+// us at 512x512x64.
+#define MM_C2R_FIELD_LENGTHS(X) X(128, 8, 16) X(256, 8, 32) X(512, 16, 32)
 
 bool field_c2r_fusable(const mm_ctx* c) {
     const mm_grid& g = c->grid;
     if (c->prec != 32 || !c->dm.on || !c->uniform || c->d_region || c->r0f.present == 0.f) return false;
     if (g.nx % 4 != 0 || 1024 % g.nx != 0 || c->dm.Lh != g.nx) return false;
     switch (c->dm.Lh) {
-#define MM_CASE(n) case n: return true;
+#define MM_CASE(m, g, q) case m: return true;
         MM_C2R_FIELD_LENGTHS(MM_CASE)
 #undef MM_CASE
         default: return false;
     }
 }
 
+// rows per CTA: as many as kC2RThreads threads transform at once, fewer on
+// small grids so that two CTAs per SM run
+static int c2r_rows(int G, long long rows) {
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const long long want = (rows + 2 * sms - 1) / (2 * sms);
+    return (int)std::max(1LL, std::min<long long>(kC2RThreads / (3 * G), want));
+}
+
 cudaError_t field_c2r_setup() {
     cudaError_t e = cudaSuccess;
-#define MM_CASE(n)                                                                                            \
-    if (e == cudaSuccess)                                                                                     \
-        e = cudaFuncSetAttribute(c2r_field_kernel<n, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
-                                 (int)c2r_field_smem<n>());                                                   \
-    if (e == cudaSuccess)                                                                                     \
-        e = cudaFuncSetAttribute(c2r_field_kernel<n, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
-                                 (int)c2r_field_smem<n>());                                                   \
-    if (e == cudaSuccess)                                                                                     \
-        e = cudaFuncSetAttribute(c2r_field_kernel<n, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                 (int)c2r_field_smem<n>());
+    const auto opt = [&](const void* k, size_t smem) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    };
+#define MM_CASE(m, g, q)                                                                                      \
+    opt((const void*)c2r_field_kernel<m, g, q, true>, c2r_field_smem<m, g, q>(kC2RThreads / (3 * g)));          \
+    opt((const void*)c2r_field_kernel<m, g, q, false>, c2r_field_smem<m, g, q>(kC2RThreads / (3 * g)));         \
+    opt((const void*)c2r_field_kernel<m, g, q, false, true>, c2r_field_smem<m, g, q>(kC2RThreads / (3 * g)));
     MM_C2R_FIELD_LENGTHS(MM_CASE)
 #undef MM_CASE
     return e;
@@ -480,20 +484,24 @@ void field_c2r_launch(mm_ctx* c, int mode, unsigned terms, const void* m, void* 
     FieldArgs<float> a = field_args<float>(c, mode, terms, (const float*)m, nullptr, (float*)out, (float*)out2,
                                            (const float*)m0, (const float*)k1, step_override, gate, kstage);
     const DemagPlan& d = c->dm;
-    C2RSpec sp{(const float2*)d.spec, (const float2*)d.tw_x, d.PyA, d.Wk};
-    const int rpc = kC2RRows;
     const long long rows = (long long)c->grid.ny * c->grid.nz;
-    const unsigned grid = (unsigned)((rows + rpc - 1) / rpc);
     const double bytes = field_bytes(c, mode, terms, false) + 3.0 * rows * (d.Kx * sizeof(float2));
     LaunchScope ls(c, "c2r_field", bytes);
     const bool quiet = field_quiet(c, mode, terms, a);
     switch (d.Lh) {
-#define MM_CASE(n)                                                                                            \
-    case n:                                                                                                   \
-        if (c->ext_terms) c2r_field_kernel<n, true><<<grid, kC2RThreads, c2r_field_smem<n>(), c->stream>>>(a, sp);      \
-        else if (quiet) c2r_field_kernel<n, false, true><<<grid, kC2RThreads, c2r_field_smem<n>(), c->stream>>>(a, sp); \
-        else c2r_field_kernel<n, false><<<grid, kC2RThreads, c2r_field_smem<n>(), c->stream>>>(a, sp);                 \
-        break;
+#define MM_CASE(M_, G_, Q_)                                                                                   \
+    case M_: {                                                                                                \
+        const int rpc = c2r_rows(G_, rows);                                                                   \
+        const C2RSpec sp{(const float2*)d.spec, (const float2*)d.tw_x, d.PyA, d.Wk, rpc};                     \
+        const unsigned grid = (unsigned)((rows + rpc - 1) / rpc);                                             \
+        const int fft = (3 * rpc * G_ + 31) / 32 * 32, cells = (rpc * c->grid.nx / 4 + 31) / 32 * 32;         \
+        const int nt = std::max(fft, std::min(kC2RThreads, cells));                                           \
+        const size_t smem = c2r_field_smem<M_, G_, Q_>(rpc);                                                  \
+        if (c->ext_terms) c2r_field_kernel<M_, G_, Q_, true><<<grid, nt, smem, c->stream>>>(a, sp);           \
+        else if (quiet) c2r_field_kernel<M_, G_, Q_, false, true><<<grid, nt, smem, c->stream>>>(a, sp);      \
+        else c2r_field_kernel<M_, G_, Q_, false><<<grid, nt, smem, c->stream>>>(a, sp);                       \
+        break;                                                                                                \
+    }
         MM_C2R_FIELD_LENGTHS(MM_CASE)
 #undef MM_CASE
         default: break;

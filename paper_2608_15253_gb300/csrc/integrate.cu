@@ -243,7 +243,7 @@ static void rk45_attempt_t(mm_ctx* c) {
     T* const* kp = (T* const*)c->d_kslot;
     const unsigned terms = c->terms;
     const bool demag = c->dm.on && (terms & MM_TERM_DEMAG);
-    const bool fused = demag && sizeof(T) == 4 && !surrogate_active(c) && demag_stage_fusable(c);
+    const bool fused = demag && !surrogate_active(c) && demag_stage_fusable(c);
     const bool fused_c2r = fused && field_c2r_fusable(c);
     for (int s = 1; s < 7; ++s) {
         if (fused_c2r) {

@@ -1,6 +1,7 @@
-"""GPU parity of the column passes at every line length that has a kernel of
+"""GPU parity of the demag passes at every line length that has a kernel of
 its own, and at both ends of the range of sizes that is padded to it: the
-middle pass of a film, of many films and of a 3-D grid, and the Y passes.
+middle pass of a film, of many films and of a 3-D grid, the Y passes and the
+X passes (with the RK45 stage state formed inside).
 The demag field is compared with the FP64 oracle's transforms; the bars are
 those of the field tests (an FP32 transform of these lengths rounds to a few
 1e-7 of the largest field, FP64 to a few 1e-16)."""
@@ -82,5 +83,52 @@ def test_many_films_match_one(n):
             for _ in range(2):
                 o.heun_step()
             assert np.abs(mm.mm_get_m(ctx, r, m.shape) - o.m).max() <= 1e-5
+    finally:
+        mm.mm_destroy(ctx)
+
+
+X_LENGTHS = [v for v in LENGTHS if v % 2 == 0 and v >= 24]
+
+
+@pytest.mark.parametrize("cells", [False, True])
+@pytest.mark.parametrize("prec", [64, 32])
+@pytest.mark.parametrize("L", X_LENGTHS)
+def test_x_passes(L, prec, cells):
+    """Rows padded to L, the smallest and the largest, even and odd; with many
+    materials the source Ms comes from the region map."""
+    mm = need_gpu()
+    from oracle.demag import demag_spectrum, h_demag
+    below = max([v for v in LENGTHS if v % 2 == 0 and v < L])
+    for nx in sorted({below // 2 + 1, L // 2 - 1, L // 2} - {1}):
+        grid = W.Grid(nx, 3, 1, 2e-9, 2e-9, 1e-9)
+        mat = W.with_cells(MAT, W.random_material_cells(grid, nx)) if cells else MAT
+        ctx = make_ctx(mm, grid, mat, precision=prec, demag=True)
+        try:
+            mm.mm_set_m(ctx, 0, W.m_random_sphere(grid, seed=nx))
+            m = mm.mm_get_m(ctx, 0, (3,) + grid.shape)
+            p = oracle_problem(grid, mat)
+            ref = np.where(p.present, h_demag(m, p, demag_spectrum(p.shape, p.d)), 0.0)
+            H = mm.mm_get_heff(ctx, 0, m.shape, TERMS["demag"])
+            assert rel_err(H, ref) < (1e-11 if prec == 64 else 5e-6)
+        finally:
+            mm.mm_destroy(ctx)
+
+
+@pytest.mark.parametrize("prec", [64, 32])
+@pytest.mark.parametrize("shape", [(33, 4, 1), (50, 3, 2), (21, 5, 2), (128, 6, 1), (171, 2, 1), (64, 40, 14)])
+def test_stage_state_formed_in_the_x_pass(shape, prec):
+    """Ten RK45 steps replayed from the oracle: rows of odd and even length,
+    one FP64 grid of more rows than take the row-per-warp kernel."""
+    mm = need_gpu()
+    from oracle.llg import Solver
+    grid = W.Grid(*shape, 2e-9, 2e-9, 2e-9)
+    m0 = W.m_random_sphere(grid, seed=7)
+    o = Solver(oracle_problem(grid, MAT), m0, dt=1e-14, rtol=1e-6)
+    dts = [o.rk45_step() for _ in range(10)]
+    ctx = make_ctx(mm, grid, MAT, precision=prec, dt=1e-14, rtol=1e-6)
+    try:
+        mm.mm_set_m(ctx, 0, m0)
+        mm.mm_step_dt(ctx, dts)
+        assert np.abs(mm.mm_get_m(ctx, 0, m0.shape) - o.m).max() <= (1e-11 if prec == 64 else 1e-5)
     finally:
         mm.mm_destroy(ctx)
