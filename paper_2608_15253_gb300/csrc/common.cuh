@@ -59,6 +59,27 @@ __device__ __forceinline__ double warp_max(double v) {
     return v;
 }
 
+// Programmatic dependent launch (launch.h): a kernel that may start before
+// its predecessor has finished calls dep_wait() before it touches anything
+// that an earlier kernel of the stream wrote (tables filled at setup may be
+// read before).  Nothing in an ordinary launch.  No kernel signals its
+// successor before its end: with an early signal the waiting CTAs cost more
+// than the shorter gap gave (512x512x64 pass 20.7 -> 25.1 ms, 64x64x16 FP64
+// 2.50 -> 3.44 ms, 128x32 FP64 3.79 -> 3.69 ms).
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// True in the one thread that calls it last over the grid, one call per block
+// (every block of the launch must call it); resets the counter for the next
+// launch.  What it reads from other blocks has to bypass L1 (__ldcg).
+__device__ __forceinline__ bool last_block(unsigned* tick) {
+    __threadfence();
+    const unsigned n = gridDim.x * gridDim.y * gridDim.z;
+    if (atomicAdd(tick, 1u) + 1u != n) return false;
+    *tick = 0;
+    __threadfence();
+    return true;
+}
+
 // Neumaier-compensated FP64 sum: value = s + c.
 struct CompSum {
     double s, c;

@@ -173,10 +173,12 @@ __global__ void __launch_bounds__(CS * G * TP, MINB) lane_conv_kernel(LaneArgs<t
         lane_commit();
     };
     int w = ST || !D3 ? blockIdx.x : blockIdx.x >> 1;             // !ST: one side of one tile per CTA
+    if (ST) dep_wait();
     if (w >= ntile) return;
     if (ST) fetch(w, 0);
-    lane_tile<N, NC, KZ, TP, NT, D3>(sk, a, w * (TP * W));
+    lane_tile<N, NC, KZ, TP, NT, D3>(sk, a, w * (TP * W));        // (the tensor is older than any launch)
     lane_commit();
+    if (!ST) dep_wait();
     for (; w < ntile; w += gridDim.x) {
 #pragma unroll 1
         for (int s = !ST && D3 ? blockIdx.x & 1 : 0; s < SIDES; ++s) {
@@ -357,8 +359,9 @@ __global__ void __launch_bounds__(3 * G * TP) lane_film_kernel(LaneArgs<typename
     lcx<N>* sm = reinterpret_cast<lcx<N>*>(smem_raw);
     N* sk = reinterpret_cast<N*>(sm + 3 * G * US);
     const int pblk = blockIdx.x * (TP * W);
-    lane_tile<N, 4, KZ, TP, NT, false>(sk, a, pblk);
+    lane_tile<N, 4, KZ, TP, NT, false>(sk, a, pblk);              // (the tensor is older than any launch)
     lane_commit();
+    dep_wait();
     const int pr = threadIdx.x % TP, t = (threadIdx.x / TP) % G, c = threadIdx.x / (G * TP);
     const int p = pblk + pr * W;
     const int o = p / a.Wk, kx = p - o * a.Wk;
@@ -471,6 +474,7 @@ __global__ void __launch_bounds__(G * TP, MINB) lane_col_kernel(LaneArgs<typenam
     const bool valid = p < a.n_cols && kx < a.Kx;
     cplx<T>* g = a.base + (valid ? (long long)o * a.o_stride + kx : 0);
     const long long ls = a.line_stride;
+    dep_wait();
     if constexpr (DIR > 0) {
         lcx<N> v[Q];
 #pragma unroll

@@ -26,6 +26,7 @@
 #include "fft_rt.cuh"
 #include "lane.h"
 #include "lane_x.cuh"
+#include "launch.h"
 
 namespace mm {
 
@@ -87,6 +88,7 @@ __device__ __forceinline__ long long spec_row(const XArgs<T>& a, int r) {
 template <typename T>
 __global__ void __launch_bounds__(256) fft_x_r2c_kernel(XArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    dep_wait();
     if (a.stage > 0 && !a.st->active) return;
     cplx<T>* sm = reinterpret_cast<cplx<T>*>(smem_raw);
     const int Lh = a.Lh;
@@ -136,6 +138,7 @@ __global__ void __launch_bounds__(256) fft_x_r2c_kernel(XArgs<T> a) {
 template <typename T>
 __global__ void __launch_bounds__(256) fft_x_c2r_kernel(XArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    dep_wait();
     cplx<T>* sm = reinterpret_cast<cplx<T>*>(smem_raw);
     const int Lh = a.Lh;
     const int pitch = Lh + 1;
@@ -240,6 +243,7 @@ __device__ __forceinline__ void tensor_multiply(const ColArgs<T>& a, cplx<T>* sm
 template <typename T, int MODE>  // MODE: +1 forward, -1 inverse, 0 convolution
 __global__ void __launch_bounds__(512) fft_col_kernel(ColArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    dep_wait();
     cplx<T>* sm = reinterpret_cast<cplx<T>*>(smem_raw);
     const int L = a.L;
     const int pitch = L + 1;
@@ -348,6 +352,7 @@ __global__ void __launch_bounds__(3 * kZT, HALF ? 5 : 4) fft_zconv_reg_kernel(ZA
     const int ky = (int)(p / a.Wk), kx = (int)(p - (long long)ky * a.Wk);
     const bool valid = ky < a.Py && kx < a.Kx;
     cplx<T>* col = a.base + c * a.comp_stride + (valid ? p : 0);
+    dep_wait();
     cplx<T> v[L];
 #pragma unroll
     for (int z = 0; z < L; ++z) v[z] = (valid && z < a.nz && (!HALF || z < L / 2)) ? col[z * a.plane] : mkc<T>(0, 0);
@@ -696,7 +701,7 @@ static void launch_x(mm_ctx* c, bool forward, const T* in, T* out_real, cplx<T>*
             // every SM (R2C of 96 or 400 rows of 128: 8.3 against 18.5 us; 3072
             // rows of 64: 24.6 against 18.5)
             LaunchScope ls(c, name, bytes);
-            (forward ? xl.fine_r2c : xl.fine_c2r)<<<rows, 32, xl.fine_line, c->stream>>>(x);
+            launch_dep(forward ? xl.fine_r2c : xl.fine_c2r, rows, 32, xl.fine_line, c, x);
             return;
         }
         // small grids: fewer rows per CTA so that two CTAs per SM run, whole warps where rows share one
@@ -704,7 +709,7 @@ static void launch_x(mm_ctx* c, bool forward, const T* in, T* out_real, cplx<T>*
         int rpc = std::max(1, (rows + 2 * sm_count() - 1) / (2 * sm_count()));
         rpc = std::min(xl.rows, (rpc + unit - 1) / unit * unit);
         LaunchScope ls(c, name, bytes);
-        (forward ? xl.r2c : xl.c2r)<<<(rows + rpc - 1) / rpc, rpc * xl.group, rpc * xl.line, c->stream>>>(x);
+        launch_dep(forward ? xl.r2c : xl.c2r, (rows + rpc - 1) / rpc, rpc * xl.group, rpc * xl.line, c, x);
         return;
     }
     int rpc = std::max(1, kMaxV * 256 / Lh);
@@ -715,7 +720,7 @@ static void launch_x(mm_ctx* c, bool forward, const T* in, T* out_real, cplx<T>*
     a.rpc = rpc;
     const int grid = (rows + rpc - 1) / rpc;
     LaunchScope ls(c, name, bytes);
-    (forward ? fft_x_r2c_kernel<T> : fft_x_c2r_kernel<T>)<<<grid, 256, smem, c->stream>>>(a);
+    launch_dep(forward ? fft_x_r2c_kernel<T> : fft_x_c2r_kernel<T>, grid, 256, smem, c, a);
 }
 
 template <typename T, int MODE>
@@ -728,7 +733,7 @@ static void launch_col(mm_ctx* c, ColArgs<T> a, int n_other, const char* name, d
     const size_t smem = (size_t)a.nc * a.TK * (a.L + 1) * sizeof(cplx<T>);
     dim3 grid((a.Kx + a.TK - 1) / a.TK, n_other);
     LaunchScope ls(c, name, bytes);
-    fft_col_kernel<T, MODE><<<grid, thr, smem, c->stream>>>(a);
+    launch_dep(fft_col_kernel<T, MODE>, grid, thr, smem, c, a);
 }
 
 // One column pass by its lane kernel: the CTAs of `sides` tiles of columns, or
@@ -744,7 +749,7 @@ static void launch_lane(mm_ctx* c, const LaneKern<T>& k, const LaneArgs<T>& a, i
         grid = std::min(tiles, std::max(1, occ) * sm_count());
     }
     LaunchScope ls(c, name, bytes);
-    k.kern<<<grid, k.threads, k.smem, c->stream>>>(a);
+    launch_dep(k.kern, grid, k.threads, k.smem, c, a);
 }
 
 // Y pass of the spectrum [3][nz][Py][Wk]; false if the length has no kernel.
@@ -884,8 +889,8 @@ static void demag_apply_t(mm_ctx* c, const T* m, T* Hd, int stage = 0, bool c2r 
             z.kc_stride = a.kc_stride; z.kk_stride = Ky * d.Wk;
             const long long cols = (long long)d.Py * d.Wk;
             LaunchScope ls(c, "fft_conv", zbytes);
-            zconv_reg_kernel(d.Pz, 2 * nz <= d.Pz)<<<(unsigned)((cols + kZT - 1) / kZT), 3 * kZT, zconv_reg_smem(d.Pz),
-                                                      c->stream>>>(z);
+            launch_dep(zconv_reg_kernel(d.Pz, 2 * nz <= d.Pz), (unsigned)((cols + kZT - 1) / kZT), 3 * kZT,
+                       zconv_reg_smem(d.Pz), c, z);
         } else if (three_d ? launch_lane_z<T>(c, S, zbytes)
                            : launch_lane_films<T>(c, d, S, ny, comp, 3 * comp, 1, "fft_conv", fbytes)) {
         } else if (three_d) {

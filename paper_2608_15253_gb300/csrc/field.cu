@@ -15,6 +15,7 @@
 #include "common.cuh"
 #include "ctx.h"
 #include "field_dev.cuh"
+#include "launch.h"
 #include "lane_x.cuh"
 
 namespace mm {
@@ -64,12 +65,7 @@ __device__ __forceinline__ void cell_store(const FieldArgs<T>& a, long long i, c
 // UNIF: one material (coefficients passed by value in the launch
 // parameters, no region map or coefficient-table loads).
 template <typename T, bool UNIF, bool EXT>
-__global__ void __launch_bounds__(256) field_kernel(FieldArgs<T> a) {
-    if (a.gate && !a.st->active) return;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if (x >= a.nx || y >= a.ny) return;
+__device__ __forceinline__ void field_cell(const FieldArgs<T>& a, int x, int y, int z) {
     const long long N = a.N;
     const long long i = ((long long)z * a.ny + y) * a.nx + x;
     const int ri = UNIF ? 0 : (a.region ? a.region[i] : 0);
@@ -90,6 +86,16 @@ __global__ void __launch_bounds__(256) field_kernel(FieldArgs<T> a) {
     v3<T> H, k;
     cell_field<T, UNIF, EXT>(a, x, y, z, i, ri, R, m, nullptr, step, H, k, a.mode != MODE_H, a.mode >= MODE_DM1);
     cell_store<T>(a, i, m, H, k);
+}
+
+template <typename T, bool UNIF, bool EXT>
+__global__ void __launch_bounds__(256) field_kernel(FieldArgs<T> a) {
+    dep_wait();
+    if (a.gate && !a.st->active) return;
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    if (x < a.nx && y < a.ny) field_cell<T, UNIF, EXT>(a, x, y, blockIdx.z);
+    if (a.tick) fixed_finish(const_cast<DevState*>(a.st), a.tick);
 }
 
 // One material, FP32, nx a multiple of V (2 or 4): each thread owns V
@@ -251,12 +257,12 @@ __device__ __forceinline__ void field_vec_cells(const FieldArgs<float>& a, int x
 
 template <int V, bool EXT, bool QUIET = false>
 __global__ void __launch_bounds__(256) field_vec_kernel(FieldArgs<float> a) {
+    dep_wait();
     if (a.gate && !a.st->active) return;
     const int x0 = V * (blockIdx.x * blockDim.x + threadIdx.x);
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if (x0 >= a.nx || y >= a.ny) return;
-    field_vec_cells<V, EXT, false, QUIET>(a, x0, y, z, nullptr, 0);
+    if (x0 < a.nx && y < a.ny) field_vec_cells<V, EXT, false, QUIET>(a, x0, y, blockIdx.z, nullptr, 0);
+    if (!QUIET && a.tick) fixed_finish(const_cast<DevState*>(a.st), a.tick);
 }
 
 // The last demag pass (inverse X, half spectrum -> real rows) fused with
@@ -284,6 +290,7 @@ constexpr size_t c2r_field_smem(int rpc) {
 template <int M, int G, int Q, bool EXT, bool QUIET = false>
 __global__ void __launch_bounds__(kC2RThreads, QUIET ? 2 : 1) c2r_field_kernel(FieldArgs<float> a, C2RSpec s) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    dep_wait();
     if (a.gate && !a.st->active) return;
     float* sH = reinterpret_cast<float*>(smem_raw);   // [rpc][3][nx], once the lines are in registers
     const int nx = a.nx, rpc = s.rpc, nrows = a.ny * a.nz;
@@ -311,6 +318,7 @@ __global__ void __launch_bounds__(kC2RThreads, QUIET ? 2 : 1) c2r_field_kernel(F
             field_vec_cells<4, EXT, true, QUIET>(a, x0, y, z, sH + rl * 3 * nx + x0, nx);
         }
     }
+    if (!QUIET && a.tick) fixed_finish(const_cast<DevState*>(a.st), a.tick);
 }
 
 constexpr int kFieldV = 4;   // cells per thread of the one-material FP32 kernel (4 measured faster than 2)
@@ -400,8 +408,9 @@ static const char* const kFieldNames[6] = {"field_H", "field_k", "field_heun1", 
 
 template <typename T>
 static void field_launch_t(mm_ctx* c, int mode, unsigned terms, const T* m, const T* Hd, T* out, T* out2,
-                           const T* m0, const T* k1, long long step_override, int gate, int kstage) {
+                           const T* m0, const T* k1, long long step_override, int gate, int kstage, bool finish) {
     FieldArgs<T> a = field_args<T>(c, mode, terms, m, Hd, out, out2, m0, k1, step_override, gate, kstage);
+    if (finish) a.tick = c->d_tick;
     const mm_grid& g = c->grid;
     dim3 blk(32, 8);
     dim3 grd((g.nx + 31) / 32, (g.ny + 7) / 8, g.nz);
@@ -410,29 +419,29 @@ static void field_launch_t(mm_ctx* c, int mode, unsigned terms, const T* m, cons
         if constexpr (sizeof(T) == 4) {
             if (g.nx % kFieldV == 0 && a.R0.present != 0.f) {
                 dim3 grdv((g.nx / kFieldV + 31) / 32, (g.ny + 7) / 8, g.nz);
-                if (c->ext_terms) field_vec_kernel<kFieldV, true><<<grdv, blk, 0, c->stream>>>(a);
+                if (c->ext_terms) launch_dep(field_vec_kernel<kFieldV, true>, grdv, blk, 0, c, a);
                 else if (field_quiet(c, mode, terms, a))
-                    field_vec_kernel<kFieldV, false, true><<<grdv, blk, 0, c->stream>>>(a);
-                else field_vec_kernel<kFieldV, false><<<grdv, blk, 0, c->stream>>>(a);
+                    launch_dep(field_vec_kernel<kFieldV, false, true>, grdv, blk, 0, c, a);
+                else launch_dep(field_vec_kernel<kFieldV, false>, grdv, blk, 0, c, a);
                 return;
             }
         }
-        if (c->ext_terms) field_kernel<T, true, true><<<grd, blk, 0, c->stream>>>(a);
-        else field_kernel<T, true, false><<<grd, blk, 0, c->stream>>>(a);
+        if (c->ext_terms) launch_dep(field_kernel<T, true, true>, grd, blk, 0, c, a);
+        else launch_dep(field_kernel<T, true, false>, grd, blk, 0, c, a);
     } else {
-        if (c->ext_terms) field_kernel<T, false, true><<<grd, blk, 0, c->stream>>>(a);
-        else field_kernel<T, false, false><<<grd, blk, 0, c->stream>>>(a);
+        if (c->ext_terms) launch_dep(field_kernel<T, false, true>, grd, blk, 0, c, a);
+        else launch_dep(field_kernel<T, false, false>, grd, blk, 0, c, a);
     }
 }
 
 void field_launch(mm_ctx* c, int mode, unsigned terms, const void* m, const void* Hd, void* out, void* out2,
-                  const void* m0, const void* k1, long long step_override, int gate, int kstage) {
+                  const void* m0, const void* k1, long long step_override, int gate, int kstage, bool finish) {
     if (c->prec == 32)
         field_launch_t<float>(c, mode, terms, (const float*)m, (const float*)Hd, (float*)out, (float*)out2,
-                              (const float*)m0, (const float*)k1, step_override, gate, kstage);
+                              (const float*)m0, (const float*)k1, step_override, gate, kstage, finish);
     else
         field_launch_t<double>(c, mode, terms, (const double*)m, (const double*)Hd, (double*)out, (double*)out2,
-                               (const double*)m0, (const double*)k1, step_override, gate, kstage);
+                               (const double*)m0, (const double*)k1, step_override, gate, kstage, finish);
 }
 
 // Inverse X pass + field kernel in one launch (FP32, one material, nx a
@@ -480,9 +489,10 @@ cudaError_t field_c2r_setup() {
 }
 
 void field_c2r_launch(mm_ctx* c, int mode, unsigned terms, const void* m, void* out, void* out2, const void* m0,
-                      const void* k1, long long step_override, int gate, int kstage) {
+                      const void* k1, long long step_override, int gate, int kstage, bool finish) {
     FieldArgs<float> a = field_args<float>(c, mode, terms, (const float*)m, nullptr, (float*)out, (float*)out2,
                                            (const float*)m0, (const float*)k1, step_override, gate, kstage);
+    if (finish) a.tick = c->d_tick;
     const DemagPlan& d = c->dm;
     const long long rows = (long long)c->grid.ny * c->grid.nz;
     const double bytes = field_bytes(c, mode, terms, false) + 3.0 * rows * (d.Kx * sizeof(float2));
@@ -497,9 +507,9 @@ void field_c2r_launch(mm_ctx* c, int mode, unsigned terms, const void* m, void* 
         const int fft = (3 * rpc * G_ + 31) / 32 * 32, cells = (rpc * c->grid.nx / 4 + 31) / 32 * 32;         \
         const int nt = std::max(fft, std::min(kC2RThreads, cells));                                           \
         const size_t smem = c2r_field_smem<M_, G_, Q_>(rpc);                                                  \
-        if (c->ext_terms) c2r_field_kernel<M_, G_, Q_, true><<<grid, nt, smem, c->stream>>>(a, sp);           \
-        else if (quiet) c2r_field_kernel<M_, G_, Q_, false, true><<<grid, nt, smem, c->stream>>>(a, sp);      \
-        else c2r_field_kernel<M_, G_, Q_, false><<<grid, nt, smem, c->stream>>>(a, sp);                       \
+        if (c->ext_terms) launch_dep(c2r_field_kernel<M_, G_, Q_, true>, grid, nt, smem, c, a, sp);           \
+        else if (quiet) launch_dep(c2r_field_kernel<M_, G_, Q_, false, true>, grid, nt, smem, c, a, sp);      \
+        else launch_dep(c2r_field_kernel<M_, G_, Q_, false>, grid, nt, smem, c, a, sp);                       \
         break;                                                                                                \
     }
         MM_C2R_FIELD_LENGTHS(MM_CASE)

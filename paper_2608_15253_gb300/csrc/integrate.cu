@@ -11,10 +11,13 @@
 // on accept m <- m5/|m5| and k7 becomes k1 (slot rotation, no copy).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "common.cuh"
 #include "ctx.h"
+#include "field_dev.cuh"
+#include "launch.h"
 
 namespace mm {
 
@@ -51,6 +54,7 @@ template <> __device__ __forceinline__ const double* err_coef<double>(const DevS
 template <typename T, int S>
 __global__ void __launch_bounds__(256) combine_kernel(const DevState* __restrict__ st, T* const* __restrict__ kptr,
                                                       const T* __restrict__ m0, T* __restrict__ ms, long long n3) {
+    dep_wait();
     if (!st->active) return;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n3) return;
@@ -71,6 +75,7 @@ __global__ void __launch_bounds__(256) combine_vec4_kernel(const DevState* __res
                                                            float* const* __restrict__ kptr,
                                                            const float* __restrict__ m0, float* __restrict__ ms,
                                                            long long n4) {
+    dep_wait();
     if (!st->active) return;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n4) return;
@@ -90,6 +95,7 @@ __global__ void __launch_bounds__(256) combine_vec4_kernel(const DevState* __res
 // per-cell error |dt sum e_j k_j|, block max, atomic max into st->err(_f)
 template <typename T>
 __global__ void error_kernel(DevState* st, T* const* __restrict__ kptr, long long N) {
+    dep_wait();
     if (!st->active) return;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const int kf = st->k_first;
@@ -125,6 +131,7 @@ __global__ void error_kernel(DevState* st, T* const* __restrict__ kptr, long lon
 
 // Start of an attempt: decide whether it runs, pick dt_eff, clear the error.
 __global__ void attempt_begin_kernel(DevState* st) {
+    dep_wait();
     const bool more = st->accepted < st->target && st->t < st->t_end && st->status == 0;
     st->active = more ? 1 : 0;
     if (!more) return;
@@ -150,6 +157,7 @@ __global__ void attempt_begin_kernel(DevState* st) {
 
 // After the error reduction: accept / reject and the next step size.
 __global__ void controller_kernel(DevState* st, int prec) {
+    dep_wait();
     st->accept = 0;
     if (!st->active) return;
     const double err = prec == 32 ? (double)st->err_f : st->err;
@@ -188,6 +196,7 @@ __global__ void controller_kernel(DevState* st, int prec) {
 template <typename T>
 __global__ void accept_kernel(const DevState* __restrict__ st, const T* __restrict__ m5, T* __restrict__ m0,
                               long long N) {
+    dep_wait();
     if (!st->active || !st->accept) return;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= N) return;
@@ -201,6 +210,7 @@ __global__ void accept_kernel(const DevState* __restrict__ st, const T* __restri
 
 // Heun step bookkeeping (fixed dt): t += dt, step += 1.
 __global__ void heun_advance_kernel(DevState* st) {
+    dep_wait();
     if (!st->active) return;
     st->t += st->dt;
     st->step += 1;
@@ -209,8 +219,26 @@ __global__ void heun_advance_kernel(DevState* st) {
 }
 
 __global__ void heun_begin_kernel(DevState* st) {
-    st->active = (st->accepted < st->target && st->t < st->t_end && st->status == 0) ? 1 : 0;
-    st->dt_eff = st->dt;
+    dep_wait();
+    fixed_begin(st);
+}
+
+// Fixed steps of a single instance: the first of a request begins here, the
+// others in the last block of the step before (256x256 film at 300 K, 8 -> 6
+// launches a step: 1.70 -> 1.65 ms for 32 steps).  The adaptive schemes keep
+// their one-thread kernels: the same bookkeeping in the last block of the
+// error and accept kernels was no faster (512x512 film 1.53 -> 1.57 ms).
+void step_begin(mm_ctx* c) {
+    if (c->batch || c->integrator == MM_RK45 || c->integrator == MM_DM_ADAPTIVE) return;
+    LaunchScope ls(c, "step_begin", 0.0);
+    launch_dep(heun_begin_kernel, 1, 1, 0, c, c->d_state);
+}
+
+// CTAs of a kernel that counts its blocks: enough to fill the chip, few
+// enough that the counter costs nothing (one atomic per 256 cells cost 50 of
+// 127 us at 512x512x64).
+static unsigned counted_blocks(long long N, unsigned tb) {
+    return (unsigned)std::min<long long>((N + tb - 1) / tb, 152 * 8);
 }
 
 void demag_eval(mm_ctx* c, const void* m, void* Hd) {
@@ -222,14 +250,14 @@ void demag_eval(mm_ctx* c, const void* m, void* Hd) {
 // grid that allows it, the last demag pass (inverse X) runs inside the
 // field kernel and H_demag never goes through global memory.
 static void demag_and_field(mm_ctx* c, bool demag, int mode, unsigned terms, const void* m, void* out, void* out2,
-                            const void* m0, const void* k1, int gate, int kstage) {
+                            const void* m0, const void* k1, int gate, int kstage, bool finish = false) {
     if (demag && !surrogate_active(c) && field_c2r_fusable(c)) {
         demag_apply_partial(c, m, 0);
-        field_c2r_launch(c, mode, terms, m, out, out2, m0, k1, -1, gate, kstage);
+        field_c2r_launch(c, mode, terms, m, out, out2, m0, k1, -1, gate, kstage, finish);
         return;
     }
     if (demag) demag_eval(c, m, c->d_hd);
-    field_launch(c, mode, terms, m, demag ? c->d_hd : nullptr, out, out2, m0, k1, -1, gate, kstage);
+    field_launch(c, mode, terms, m, demag ? c->d_hd : nullptr, out, out2, m0, k1, -1, gate, kstage, finish);
 }
 
 template <typename T>
@@ -238,7 +266,7 @@ static void rk45_attempt_t(mm_ctx* c) {
     const unsigned tb = 256, nb3 = (unsigned)((n3 + tb - 1) / tb), nb = (unsigned)((N + tb - 1) / tb);
     {
         LaunchScope ls(c, "rk_begin", 0.0);
-        attempt_begin_kernel<<<1, 1, 0, c->stream>>>(c->d_state);
+        launch_dep(attempt_begin_kernel, 1, 1, 0, c, c->d_state);
     }
     T* const* kp = (T* const*)c->d_kslot;
     const unsigned terms = c->terms;
@@ -266,13 +294,13 @@ static void rk45_attempt_t(mm_ctx* c) {
                         nullptr, combine_vec4_kernel<1>, combine_vec4_kernel<2>, combine_vec4_kernel<3>,
                         combine_vec4_kernel<4>, combine_vec4_kernel<5>, combine_vec4_kernel<6>};
                     const long long n4 = n3 / 4;
-                    k4[s]<<<(unsigned)((n4 + tb - 1) / tb), tb, 0, c->stream>>>(
-                        c->d_state, (float* const*)kp, (const float*)c->d_m, (float*)c->d_mtmp, n4);
+                    launch_dep(k4[s], (unsigned)((n4 + tb - 1) / tb), tb, 0, c, c->d_state, (float* const*)kp,
+                               (const float*)c->d_m, (float*)c->d_mtmp, n4);
                 } else {
-                    kern[s]<<<nb3, tb, 0, c->stream>>>(c->d_state, kp, (const T*)c->d_m, (T*)c->d_mtmp, n3);
+                    launch_dep(kern[s], nb3, tb, 0, c, c->d_state, kp, (const T*)c->d_m, (T*)c->d_mtmp, n3);
                 }
             } else {
-                kern[s]<<<nb3, tb, 0, c->stream>>>(c->d_state, kp, (const T*)c->d_m, (T*)c->d_mtmp, n3);
+                launch_dep(kern[s], nb3, tb, 0, c, c->d_state, kp, (const T*)c->d_m, (T*)c->d_mtmp, n3);
             }
         }
         if (demag && !fused) demag_eval(c, c->d_mtmp, c->d_hd);
@@ -283,15 +311,15 @@ static void rk45_attempt_t(mm_ctx* c) {
     }
     {
         LaunchScope ls(c, "rk_error", (double)sizeof(T) * 3 * N * 6);
-        error_kernel<T><<<nb, tb, 0, c->stream>>>(c->d_state, kp, N);
+        launch_dep(error_kernel<T>, nb, tb, 0, c, c->d_state, kp, N);
     }
     {
         LaunchScope ls(c, "rk_control", 0.0);
-        controller_kernel<<<1, 1, 0, c->stream>>>(c->d_state, c->prec);
+        launch_dep(controller_kernel, 1, 1, 0, c, c->d_state, c->prec);
     }
     {
         LaunchScope ls(c, "rk_accept", (double)sizeof(T) * 6 * N);
-        accept_kernel<T><<<nb, tb, 0, c->stream>>>(c->d_state, (const T*)c->d_mtmp, (T*)c->d_m, N);
+        launch_dep(accept_kernel<T>, nb, tb, 0, c, c->d_state, (const T*)c->d_mtmp, (T*)c->d_m, N);
     }
 }
 
@@ -308,12 +336,12 @@ void rk45_first_slope(mm_ctx* c) {
 
 void heun_batch_begin(mm_ctx* c) {
     LaunchScope ls(c, "heun_begin", 0.0);
-    heun_begin_kernel<<<1, 1, 0, c->stream>>>(c->d_state);
+    launch_dep(heun_begin_kernel, 1, 1, 0, c, c->d_state);
 }
 
 void heun_batch_advance(mm_ctx* c) {
     LaunchScope ls(c, "heun_advance", 0.0);
-    heun_advance_kernel<<<1, 1, 0, c->stream>>>(c->d_state);
+    launch_dep(heun_advance_kernel, 1, 1, 0, c, c->d_state);
 }
 
 // Classical RK4 (Methods, "Integrators": fixed step): stage states
@@ -323,6 +351,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) rk4_stage_kernel(const DevState* __restrict__ st, const T* __restrict__ m0,
                                                         const T* __restrict__ k, double c, T* __restrict__ out,
                                                         long long n3) {
+    dep_wait();
     if (!st->active) return;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n3) return;
@@ -331,24 +360,26 @@ __global__ void __launch_bounds__(256) rk4_stage_kernel(const DevState* __restri
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) rk4_final_kernel(const DevState* __restrict__ st, T* __restrict__ m0,
+__global__ void __launch_bounds__(256) rk4_final_kernel(DevState* st, T* __restrict__ m0,
                                                         const T* __restrict__ k1, const T* __restrict__ k2,
                                                         const T* __restrict__ k3, const T* __restrict__ k4,
-                                                        long long N) {
+                                                        long long N, unsigned* tick) {
+    dep_wait();
     if (!st->active) return;
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= N) return;
     const T h6 = (T)(st->dt / 6.0);
-    T v[3];
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+        T v[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const long long j = c * N + i;
-        v[c] = m0[j] + h6 * (k1[j] + (T)2 * k2[j] + (T)2 * k3[j] + k4[j]);
+        for (int c = 0; c < 3; ++c) {
+            const long long j = c * N + i;
+            v[c] = m0[j] + h6 * (k1[j] + (T)2 * k2[j] + (T)2 * k3[j] + k4[j]);
+        }
+        const T n2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+        const T inv = n2 > (T)0 ? (T)1 / sqrt(n2) : (T)0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) m0[c * N + i] = v[c] * inv;
     }
-    const T n2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-    const T inv = n2 > (T)0 ? (T)1 / sqrt(n2) : (T)0;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) m0[c * N + i] = v[c] * inv;
+    fixed_finish(st, tick);
 }
 
 template <typename T>
@@ -356,29 +387,23 @@ static void rk4_step_t(mm_ctx* c) {
     const unsigned terms = c->terms;
     const bool demag = c->dm.on && (terms & MM_TERM_DEMAG);
     const long long N = c->N, n3 = 3 * N;
-    const unsigned tb = 256, nb3 = (unsigned)((n3 + tb - 1) / tb), nb = (unsigned)((N + tb - 1) / tb);
-    {
-        LaunchScope ls(c, "rk4_begin", 0.0);
-        heun_begin_kernel<<<1, 1, 0, c->stream>>>(c->d_state);
-    }
+    const unsigned tb = 256, nb3 = (unsigned)((n3 + tb - 1) / tb);
     static const double cs[4] = {0.0, 0.5, 0.5, 1.0};
     for (int s = 0; s < 4; ++s) {
         const void* ms = c->d_m;
         if (s > 0) {
             LaunchScope ls(c, "rk4_stage", (double)sizeof(T) * n3 * 3);
-            rk4_stage_kernel<T><<<nb3, tb, 0, c->stream>>>(c->d_state, (const T*)c->d_m, (const T*)c->d_k[s - 1],
-                                                            cs[s], (T*)c->d_mtmp, n3);
+            launch_dep(rk4_stage_kernel<T>, nb3, tb, 0, c, c->d_state, (const T*)c->d_m, (const T*)c->d_k[s - 1],
+                       cs[s], (T*)c->d_mtmp, n3);
             ms = c->d_mtmp;
         }
         demag_and_field(c, demag, MODE_K, terms, ms, c->d_k[s], nullptr, nullptr, nullptr, 1, 0);
     }
     {
         LaunchScope ls(c, "rk4_final", (double)sizeof(T) * N * 18);
-        rk4_final_kernel<T><<<nb, tb, 0, c->stream>>>(c->d_state, (T*)c->d_m, (const T*)c->d_k[0], (const T*)c->d_k[1],
-                                                       (const T*)c->d_k[2], (const T*)c->d_k[3], N);
+        launch_dep(rk4_final_kernel<T>, counted_blocks(N, tb), tb, 0, c, c->d_state, (T*)c->d_m,
+                   (const T*)c->d_k[0], (const T*)c->d_k[1], (const T*)c->d_k[2], (const T*)c->d_k[3], N, c->d_tick);
     }
-    LaunchScope ls(c, "rk4_advance", 0.0);
-    heun_advance_kernel<<<1, 1, 0, c->stream>>>(c->d_state);
 }
 
 void rk4_step(mm_ctx* c) {
@@ -389,16 +414,10 @@ void rk4_step(mm_ctx* c) {
 void heun_step(mm_ctx* c) {
     const unsigned terms = c->terms;
     const bool demag = c->dm.on && (terms & MM_TERM_DEMAG);
-    {
-        LaunchScope ls(c, "heun_begin", 0.0);
-        heun_begin_kernel<<<1, 1, 0, c->stream>>>(c->d_state);
-    }
     // predictor: k1 = f(m, H(m) + H_th); m* = m + dt k1
     demag_and_field(c, demag, MODE_HEUN1, terms, c->d_m, c->d_mtmp, c->d_k[0], nullptr, nullptr, 1, 0);
     // corrector: m' = normalise(m + dt/2 (k1 + f(m*, H(m*) + H_th))), same noise
-    demag_and_field(c, demag, MODE_HEUN2, terms, c->d_mtmp, c->d_m, nullptr, c->d_m, c->d_k[0], 1, 0);
-    LaunchScope ls(c, "heun_advance", 0.0);
-    heun_advance_kernel<<<1, 1, 0, c->stream>>>(c->d_state);
+    demag_and_field(c, demag, MODE_HEUN2, terms, c->d_mtmp, c->d_m, nullptr, c->d_m, c->d_k[0], 1, 0, true);
 }
 
 // Depondt-Mertens (Methods, "Integrators"): Omega_1 = Omega(m) and the
@@ -410,20 +429,15 @@ void heun_step(mm_ctx* c) {
 void dm_step(mm_ctx* c) {
     const unsigned terms = c->terms;
     const bool demag = c->dm.on && (terms & MM_TERM_DEMAG);
-    {
-        LaunchScope ls(c, "dm_begin", 0.0);
-        heun_begin_kernel<<<1, 1, 0, c->stream>>>(c->d_state);
-    }
     demag_and_field(c, demag, MODE_DM1, terms, c->d_m, c->d_mtmp, c->d_k[0], nullptr, nullptr, 1, 0);
-    demag_and_field(c, demag, MODE_DM2, terms, c->d_mtmp, c->d_m, nullptr, c->d_m, c->d_k[0], 1, 0);
-    LaunchScope ls(c, "dm_advance", 0.0);
-    heun_advance_kernel<<<1, 1, 0, c->stream>>>(c->d_state);
+    demag_and_field(c, demag, MODE_DM2, terms, c->d_mtmp, c->d_m, nullptr, c->d_m, c->d_k[0], 1, 0, true);
 }
 
 // Adaptive Depondt-Mertens: err = max over cells |cand - m*| (the corrector
 // against the first-order predictor), block max, atomic max into st->err(_f).
 template <typename T>
 __global__ void dm_error_kernel(DevState* st, const T* __restrict__ cand, const T* __restrict__ mstar, long long N) {
+    dep_wait();
     if (!st->active) return;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     T e2 = 0;
@@ -457,20 +471,20 @@ static void dm_adaptive_attempt_t(mm_ctx* c) {
     const unsigned tb = 256, nb = (unsigned)((N + tb - 1) / tb);
     {
         LaunchScope ls(c, "dm_begin", 0.0);
-        attempt_begin_kernel<<<1, 1, 0, c->stream>>>(c->d_state);
+        launch_dep(attempt_begin_kernel, 1, 1, 0, c, c->d_state);
     }
     demag_and_field(c, demag, MODE_DM1, terms, c->d_m, c->d_mtmp, c->d_k[0], nullptr, nullptr, 1, 0);
     demag_and_field(c, demag, MODE_DM2, terms, c->d_mtmp, c->d_k[1], nullptr, c->d_m, c->d_k[0], 1, 0);
     {
         LaunchScope ls(c, "dm_error", (double)sizeof(T) * 6 * N);
-        dm_error_kernel<T><<<nb, tb, 0, c->stream>>>(c->d_state, (const T*)c->d_k[1], (const T*)c->d_mtmp, N);
+        launch_dep(dm_error_kernel<T>, nb, tb, 0, c, c->d_state, (const T*)c->d_k[1], (const T*)c->d_mtmp, N);
     }
     {
         LaunchScope ls(c, "dm_control", 0.0);
-        controller_kernel<<<1, 1, 0, c->stream>>>(c->d_state, c->prec);
+        launch_dep(controller_kernel, 1, 1, 0, c, c->d_state, c->prec);
     }
     LaunchScope ls(c, "dm_accept", (double)sizeof(T) * 6 * N);
-    accept_kernel<T><<<nb, tb, 0, c->stream>>>(c->d_state, (const T*)c->d_k[1], (T*)c->d_m, N);
+    launch_dep(accept_kernel<T>, nb, tb, 0, c, c->d_state, (const T*)c->d_k[1], (T*)c->d_m, N);
 }
 
 void dm_adaptive_attempt(mm_ctx* c) {

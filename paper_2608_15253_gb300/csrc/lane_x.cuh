@@ -160,6 +160,7 @@ template <typename T, int M, int G, int Q, int ROWS>
 __global__ void __launch_bounds__(G* ROWS) lane_r2c_kernel(XLaneArgs<T> a) {
     using S = XSplit<M, G, Q>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    dep_wait();
     if (a.stage > 0 && !a.st->active) return;
     const int t = threadIdx.x % G, rl = threadIdx.x / G;
     lcx<T>* sm = reinterpret_cast<lcx<T>*>(smem_raw) + rl * S::LINE;
@@ -287,6 +288,7 @@ template <typename T, int M, int G, int Q, int ROWS>
 __global__ void __launch_bounds__(G* ROWS) lane_c2r_kernel(XLaneArgs<T> a) {
     using S = XSplit<M, G, Q>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    dep_wait();
     const int t = threadIdx.x % G, rl = threadIdx.x / G;
     lcx<T>* sm = reinterpret_cast<lcx<T>*>(smem_raw) + rl * S::LINE;
     const int row = blockIdx.x * (blockDim.x / G) + rl;
@@ -378,6 +380,7 @@ __device__ __forceinline__ void fine_passes(lcx<T>* sm, const cplx<T>* __restric
 template <typename T, int M>
 __global__ void __launch_bounds__(128) fine_r2c_kernel(XLaneArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    dep_wait();
     if (a.stage > 0 && !a.st->active) return;
     lcx<T>* sm = reinterpret_cast<lcx<T>*>(smem_raw) + (threadIdx.x >> 5) * fine_line(M);
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -421,6 +424,7 @@ __global__ void __launch_bounds__(128) fine_r2c_kernel(XLaneArgs<T> a) {
 template <typename T, int M>
 __global__ void __launch_bounds__(128) fine_c2r_kernel(XLaneArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    dep_wait();
     lcx<T>* sm = reinterpret_cast<lcx<T>*>(smem_raw) + (threadIdx.x >> 5) * fine_line(M);
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= a.rows) return;                                    // whole warp
