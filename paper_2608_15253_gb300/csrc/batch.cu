@@ -44,6 +44,7 @@ struct BatchHost {
     double sigma_V = 1.0;   // cell volume used in the thermal scale
     bool macro = false;     // every replica one cell, no demag: macro_kernel
     bool tile = false;      // no demag, every replica at most kTileMaxCells cells: tile_kernel
+    bool tile_demag = false;   // one small size class with demag: tile_demag_kernel in the stacked shape
     int nmax = 0;           // largest replica (cells)
     // retire/refill
     bool trials_on = false;
@@ -214,7 +215,9 @@ mm_status batch_setup(mm_ctx* c, BatchHost* b, const std::vector<mm_grid>& grids
         e = cudaMalloc(&b->d_scratch, sizeof(float2) * b->scratch_stride * max_blocks);
         if (e != cudaSuccess) return cuda_check(c, e, "batch scratch");
     }
+    b->tile_demag = demag && b->cls.size() == 1 && tile_demag_supported(b->cls[0].Lh, b->cls[0].Py);
     e = batch_kernel_attributes_256();
+    if (e == cudaSuccess && b->tile_demag) e = tile_demag_attributes(b->cls[0].Lh, b->cls[0].Py);
     if (e == cudaSuccess) e = batch_kernel_attributes_512();
     return cuda_check(c, e, "batch kernel attributes");
 }
@@ -289,7 +292,9 @@ static void launch_stage(mm_ctx* c, BatchHost* b, int stage) {
     else batch_kernel_launch_256(a, b->blocks, b->smem, c->stream);
 }
 
-bool batch_is_fused(BatchHost* b) { return b->macro || b->tile; }
+// Small films with demag are fused in the stacked shape, which the autotuner
+// picks for them; the persistent shape stays what the caller asked for.
+bool batch_is_fused(BatchHost* b) { return b->macro || b->tile || (b->tile_demag && b->stacked); }
 
 // one launch of `nsteps` fused steps of every replica (one-cell or small
 // films without demag), then the step bookkeeping
@@ -314,7 +319,8 @@ void batch_macro_steps(mm_ctx* c, BatchHost* b, int nsteps) {
         double cells = 0;
         for (const RepDev& r : b->rep) cells += (double)r.nx * r.ny;
         LaunchScope ls(c, "tile_steps", cells * 24.0);
-        tile_kernel_launch(a, c->stream);
+        if (b->tile) tile_kernel_launch(a, c->stream);
+        else tile_demag_launch(a, b->d_cls, b->cls[0].Lh, b->cls[0].Py, c->stream);
     }
     LaunchScope ls(c, "macro_advance", 0.0);
     macro_advance_launch(c->d_state, nsteps, c->stream);

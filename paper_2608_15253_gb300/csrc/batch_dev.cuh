@@ -464,6 +464,10 @@ void stacked_trials_launch(const BatchArgs& a, int R, cudaStream_t s);
 void macro_kernel_launch(const MacroArgs& a, cudaStream_t s);
 void tile_kernel_launch(const MacroArgs& a, cudaStream_t s);
 cudaError_t tile_kernel_attributes();
+// batch_tile.cu: small films with demag, by half length and column length
+bool tile_demag_supported(int Lh, int Py);
+cudaError_t tile_demag_attributes(int Lh, int Py);
+void tile_demag_launch(const MacroArgs& a, const ClsDev* cls, int Lh, int Py, cudaStream_t s);
 void macro_advance_launch(DevState* st, int nsteps, cudaStream_t s);
 
 // host wrappers, one set per instantiated thread count

@@ -106,16 +106,16 @@ __device__ __forceinline__ void x_merge(cplx<T> xk, cplx<T> xm, cplx<T> w, lcx<T
 
 // Half spectrum X[0..M] of one row to the pairs of its real values:
 // store(n, (x[2n], x[2n+1])) for n = q G + t, q < QIN.  sm: the row's LINE
-// values; taken() runs when they are in registers.
-template <typename T, int M, int G, int Q, typename Taken, typename Store>
-__device__ __forceinline__ void lane_c2r_row(const cplx<T>* __restrict__ X, const cplx<T>* __restrict__ tw, lcx<T>* sm,
+// values; taken() runs when they are in registers.  INPLACE: X lies where sm
+// does (the rows of a warp; no store to a row that is not valid).
+template <typename T, int M, int G, int Q, bool INPLACE = false, typename Taken, typename Store>
+__device__ __forceinline__ void lane_c2r_row(const cplx<T>* X, const cplx<T>* __restrict__ tw, lcx<T>* sm,
                                              int t, bool valid, Taken taken, Store store) {
     using S = XSplit<M, G, Q>;
-#pragma unroll
-    for (int i = 0; i < S::NSL; ++i) {
+    static_assert(!INPLACE || S::WARP, "in place: rows within warps");
+    lcx<T> zks[INPLACE ? S::NSL : 1][G + 1], zms[INPLACE ? S::NSL : 1][G + 1];
+    auto gather = [&](int i, lcx<T>* zk, lcx<T>* zm) {
         const int j = t + i * G;
-        if (S::NS % G != 0 && j >= S::NS) continue;
-        lcx<T> zk[G + 1], zm[G + 1];
 #pragma unroll
         for (int e = 0; e < (i == 0 ? (S::NE > G ? S::NE : G) : G); ++e) {
             int k = j + Q * e;
@@ -126,6 +126,21 @@ __device__ __forceinline__ void lane_c2r_row(const cplx<T>* __restrict__ X, cons
             if (valid) { xk = X[k]; xm = X[M - k]; }
             x_merge<T>(xk, xm, __ldg(tw + k), zk[e], zm[e]);
         }
+    };
+    if constexpr (INPLACE) {
+#pragma unroll
+        for (int i = 0; i < S::NSL; ++i)
+            if (t + i * G < S::NS) gather(i, zks[i], zms[i]);
+        __syncwarp();                                             // every value of the spectrum is in registers
+    }
+#pragma unroll
+    for (int i = 0; i < S::NSL; ++i) {
+        const int j = t + i * G;
+        if (S::NS % G != 0 && j >= S::NS) continue;
+        lcx<T>* zk = zks[INPLACE ? i : 0];
+        lcx<T>* zm = zms[INPLACE ? i : 0];
+        if (!INPLACE) gather(i, zk, zm);
+        if (INPLACE && !valid) continue;
         lcx<T> a[G], b[G];
 #pragma unroll
         for (int x = 0; x < G; ++x) {

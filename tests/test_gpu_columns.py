@@ -132,3 +132,41 @@ def test_stage_state_formed_in_the_x_pass(shape, prec):
         assert np.abs(mm.mm_get_m(ctx, 0, m0.shape) - o.m).max() <= (1e-11 if prec == 64 else 1e-5)
     finally:
         mm.mm_destroy(ctx)
+
+
+@pytest.mark.parametrize("integrator", ["heun", "dm"])
+@pytest.mark.parametrize("n", [(8, 8), (7, 8), (12, 12), (16, 16), (15, 16), (16, 15), (24, 24), (32, 32), (31, 32)])
+def test_small_film_ensembles_match_oracle(n, integrator):
+    """Films of one small size in the stacked shape (a block of steps per
+    launch): the whole range of the sizes it takes, a temperature and a current
+    per replica, 12 steps against the FP64 oracle."""
+    mm = need_gpu()
+    from oracle.llg import Solver, Torque
+    nx, ny = n
+    R, cell = 5, (2e-9, 2e-9, 1e-9)
+    mat = W.Material(Ms=1.1e6, A=2e-11, alpha=0.05, Ku1=9e5, D=1e-3)
+    M = mm.Material(mat.Ms, mat.A, mat.alpha, mat.Ku1, mat.u, mat.D)
+    cfg = mm.make_config(precision=32, integrator=mm.MM_HEUN if integrator == "heun" else mm.MM_DM,
+                         demag=mm.MM_DEMAG_EXACT, dt=1e-14)
+    seeds = np.arange(1, R + 1, dtype=np.uint64) * np.uint64(7919)
+    T, J = np.linspace(0.0, 400.0, R), np.linspace(1e11, 3e11, R)
+    ctx = mm.mm_create_batch([mm.make_grid(nx, ny, 1, *cell)] * R, M.s, cfg, seeds)
+    try:
+        mm.mm_batch_set_shape(ctx, 0)
+        mm.mm_set_temperature(ctx, T)
+        mm.mm_set_torque(ctx, mm.make_torque(mm.MM_TORQUE_SOT, p=(0, 1, 0), theta_SH=0.1, fl_ratio=0.3), J)
+        g = W.Grid(nx, ny, 1, *cell)
+        m0 = [W.m_perp(g, seed=100 + r, tilt=0.3) for r in range(R)]
+        for r in range(R):
+            mm.mm_set_m(ctx, r, m0[r])
+        mm.mm_step(ctx, 7)
+        mm.mm_step(ctx, 5)
+        for r in range(R):
+            o = Solver(oracle_problem(g, mat), m0[r], terms=("exchange", "dmi", "anisotropy", "zeeman", "demag"), T=T[r],
+                       seed=int(seeds[r]), dt=1e-14,
+                       torque=Torque(kind="sot", J=J[r], p=(0, 1, 0), theta_SH=0.1, fl_ratio=0.3))
+            for _ in range(12):
+                o.heun_step() if integrator == "heun" else o.dm_step()
+            assert np.abs(mm.mm_get_m(ctx, r, m0[r].shape) - o.m).max() <= 1e-5, (r, n)
+    finally:
+        mm.mm_destroy(ctx)
