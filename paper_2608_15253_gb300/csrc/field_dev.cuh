@@ -289,18 +289,26 @@ __device__ __forceinline__ void sincos_t(double x, double* s, double* c) { sinco
 //   m + s (w x m) + q (w (w.m) - |w|^2 m),  s = sin(a) / |w|,
 //   q = (1 - cos a) / |w|^2,
 // with sin a = 2 sin(a/2) cos(a/2) and 1 - cos a = 2 sin^2(a/2) from one
-// half-angle sincos; for a^2 < 1e-6 (w = 0 included) the Taylor series
-// sin(a)/a = 1 - a^2/6 + a^4/120 and (1 - cos a)/a^2 = 1/2 - a^2/24 + a^4/720
-// (next terms below 1e-21).  For constant w this is the exact solution of
-// dm/dt = w x m over dt.
+// half-angle sincos.  Small angles (w = 0 included) take the Taylor series of
+// sin(a)/a and (1 - cos a)/a^2 in a^2: in FP64 below a^2 = 1e-6 to the third
+// term (the next is below 1e-21), in FP32 below a = 1/2 to the fifth (the next
+// is below 3e-11), which is every step of the usual sizes: a few fused
+// multiply-adds in place of a square root, a sincos and two divisions, and a
+// rounding closer (7e-8 against 2e-7).  For constant w this is the exact
+// solution of dm/dt = w x m over dt.
 template <typename T>
 __device__ __forceinline__ v3<T> rodrigues(const v3<T>& m, const v3<T>& w, T dt) {
     const T w2 = dot(w, w);
     const T a2 = w2 * dt * dt;
     T s, q;
-    if (a2 < (T)1e-6) {
-        s = dt * ((T)1 - a2 * ((T)(1.0 / 6.0) - a2 * (T)(1.0 / 120.0)));
-        q = dt * dt * ((T)0.5 - a2 * ((T)(1.0 / 24.0) - a2 * (T)(1.0 / 720.0)));
+    if (sizeof(T) == 4 ? a2 < (T)0.25 : a2 < (T)1e-6) {
+        if (sizeof(T) == 4) {
+            s = dt * ((T)1 - a2 * ((T)(1.0 / 6.0) - a2 * ((T)(1.0 / 120.0) - a2 * ((T)(1.0 / 5040.0) - a2 * (T)(1.0 / 362880.0)))));
+            q = dt * dt * ((T)0.5 - a2 * ((T)(1.0 / 24.0) - a2 * ((T)(1.0 / 720.0) - a2 * ((T)(1.0 / 40320.0) - a2 * (T)(1.0 / 3628800.0)))));
+        } else {
+            s = dt * ((T)1 - a2 * ((T)(1.0 / 6.0) - a2 * (T)(1.0 / 120.0)));
+            q = dt * dt * ((T)0.5 - a2 * ((T)(1.0 / 24.0) - a2 * (T)(1.0 / 720.0)));
+        }
     } else {
         const T a = sqrt(a2);
         T sh, ch;
