@@ -412,17 +412,23 @@ static void field_launch_t(mm_ctx* c, int mode, unsigned terms, const T* m, cons
     FieldArgs<T> a = field_args<T>(c, mode, terms, m, Hd, out, out2, m0, k1, step_override, gate, kstage);
     if (finish) a.tick = c->d_tick;
     const mm_grid& g = c->grid;
-    dim3 blk(32, 8);
-    dim3 grd((g.nx + 31) / 32, (g.ny + 7) / 8, g.nz);
+    // rows of 32 cells per warp, eight warps to a CTA; on small grids fewer, so
+    // that every scheduler gets a warp (FP64, 128x32: 15.4 -> 10.7 us; 16 CTAs of
+    // eight warps left the other SMs' FP64 pipes idle)
+    const bool vec = sizeof(T) == 4 && c->uniform && !a.region && g.nx % kFieldV == 0 && a.R0.present != (T)0;
+    const int gx = vec ? (g.nx / kFieldV + 31) / 32 : (g.nx + 31) / 32;
+    int by = 8;
+    while (by > 1 && (long long)gx * ((g.ny + by - 1) / by) * g.nz < 4 * 152) by /= 2;
+    dim3 blk(32, by);
+    dim3 grd(gx, (g.ny + by - 1) / by, g.nz);
     LaunchScope ls(c, kFieldNames[mode], field_bytes(c, mode, terms, Hd != nullptr));
     if (c->uniform && !a.region) {
         if constexpr (sizeof(T) == 4) {
-            if (g.nx % kFieldV == 0 && a.R0.present != 0.f) {
-                dim3 grdv((g.nx / kFieldV + 31) / 32, (g.ny + 7) / 8, g.nz);
-                if (c->ext_terms) launch_dep(field_vec_kernel<kFieldV, true>, grdv, blk, 0, c, a);
+            if (vec) {
+                if (c->ext_terms) launch_dep(field_vec_kernel<kFieldV, true>, grd, blk, 0, c, a);
                 else if (field_quiet(c, mode, terms, a))
-                    launch_dep(field_vec_kernel<kFieldV, false, true>, grdv, blk, 0, c, a);
-                else launch_dep(field_vec_kernel<kFieldV, false>, grdv, blk, 0, c, a);
+                    launch_dep(field_vec_kernel<kFieldV, false, true>, grd, blk, 0, c, a);
+                else launch_dep(field_vec_kernel<kFieldV, false>, grd, blk, 0, c, a);
                 return;
             }
         }

@@ -40,7 +40,7 @@ template <typename T> struct XLaneArgs;
 
 template <typename T>
 struct XLane {
-    void (*r2c)(XLaneArgs<T>) = nullptr;
+    void (*r2c[3])(XLaneArgs<T>) = {};          // by XInput: plain rows, stage state, anything
     void (*c2r)(XLaneArgs<T>) = nullptr;
     int group = 0, rows = 0;
     size_t line = 0;
@@ -48,6 +48,14 @@ struct XLane {
     void (*fine_c2r)(XLaneArgs<T>) = nullptr;
     size_t fine_line = 0;
 };
+
+// Middle pass of one FP64 film in the row-per-warp passes (lane_x.cuh).
+template <typename T> struct FineFilmArgs;
+struct FineFilm {
+    void (*kern)(FineFilmArgs<double>) = nullptr;
+    size_t smem = 0;
+};
+FineFilm fine_film(int L);
 
 // (M, G, Q, rows): the slots of a row, Q/2, fill its G threads evenly where
 // the length allows it (Q = 2 G or a multiple), about 128 threads per CTA
@@ -58,6 +66,9 @@ struct XLane {
     X(384, 16, 24, 8) X(432, 16, 27, 8) X(486, 18, 27, 7) X(512, 16, 32, 8)
 
 template <typename T> XLane<T> lane_x(int M);
+// the third of the r2c kernels, in a translation unit of its own
+void (*lane_r2c_any_f(int M))(XLaneArgs<float>);
+void (*lane_r2c_any_d(int M))(XLaneArgs<double>);
 template <> XLane<float> lane_x<float>(int M);
 template <> XLane<double> lane_x<double>(int M);
 

@@ -3,6 +3,7 @@
 // every SM's FP64 units (two fused multiply-adds per clock each).
 #include "conv_lane.cuh"
 #include "lane.h"
+#include "lane_x.cuh"
 
 namespace mm {
 
@@ -14,6 +15,15 @@ namespace mm {
 template <> LaneKern<double> lane_film<double>(int L) {
     switch (L) {
 #define MM_CASE(l, g, q) case l: return {lane_film_kernel<double, l, g, q, 2>, 3 * g * 2, 2, lane_film_smem<double, l, g, q, 2>(), false};
+        MM_FILM_D(MM_CASE)
+#undef MM_CASE
+        default: return {};
+    }
+}
+
+FineFilm fine_film(int L) {
+    switch (L) {
+#define MM_CASE(l, g, q) case l: return {fine_film_kernel<double, l>, 3 * fine_line(l) * sizeof(lcx<double>)};
         MM_FILM_D(MM_CASE)
 #undef MM_CASE
         default: return {};

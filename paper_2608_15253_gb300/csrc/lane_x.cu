@@ -1,10 +1,14 @@
 // X passes of FP32 rows (lane_x.cuh): shapes by half length M = G * Q.  One
 // GB300, forward pass with the RK45 stage formed in it, mean of the stages:
-//   512x512x64  285 us against 380 for a row per warp in radix-8 passes
-//               (6.4 TB/s: what the slopes and the spectrum cost)
-//   250x250x40  63 us against 71;  150x150x24 with a region map 20 us against
-//               43 plus 10 for the stage state formed by a kernel of its own
-// inverse: 150x150x24 11.4 us against 29, 250x250x40 35 against 39.
+//   512x512x64  239 us against 380 for a row per warp in radix-8 passes
+//   250x250x40  52 us against 71;  256x256x16 24 us against 32
+//   150x150x24 with a region map 20 us against 43 plus 10 for the stage state
+//   formed by a kernel of its own
+// inverse: 150x150x24 11.5 us against 29, 250x250x40 35 against 39.
+// The straight-line code of a row is long; the kernels are kept to one body
+// per kind of row without branches in the split (with a body per stage and
+// the general rows in the same kernel: 285, 63 and 33 us, half of a small
+// grid's time in instruction fetches).
 #include "lane.h"
 #include "lane_x.cuh"
 
@@ -13,7 +17,8 @@ namespace mm {
 template <> XLane<float> lane_x<float>(int M) {
     switch (M) {
 #define MM_CASE(m, g, q, rows) \
-    case m: return {lane_r2c_kernel<float, m, g, q, rows>, lane_c2r_kernel<float, m, g, q, rows>, g, rows, XSplit<m, g, q>::LINE * sizeof(lcx<float>)};
+    case m: return {{lane_r2c_kernel<float, m, g, q, rows, X_PLAIN>, lane_r2c_kernel<float, m, g, q, rows, X_STAGE>, lane_r2c_any_f(m)}, \
+                    lane_c2r_kernel<float, m, g, q, rows>, g, rows, XSplit<m, g, q>::LINE * sizeof(lcx<float>)};
         MM_XLANE_SHAPES(MM_CASE)
 #undef MM_CASE
         default: return {};

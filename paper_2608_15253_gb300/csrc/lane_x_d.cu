@@ -10,7 +10,8 @@ namespace mm {
 template <> XLane<double> lane_x<double>(int M) {
     switch (M) {
 #define MM_CASE(m, g, q, rows) \
-    case m: return {lane_r2c_kernel<double, m, g, q, rows>, lane_c2r_kernel<double, m, g, q, rows>, g, rows, XSplit<m, g, q>::LINE * sizeof(lcx<double>), \
+    case m: return {{lane_r2c_kernel<double, m, g, q, rows, X_PLAIN>, lane_r2c_kernel<double, m, g, q, rows, X_STAGE>, lane_r2c_any_d(m)}, \
+                    lane_c2r_kernel<double, m, g, q, rows>, g, rows, XSplit<m, g, q>::LINE * sizeof(lcx<double>), \
                     fine_r2c_kernel<double, m>, fine_c2r_kernel<double, m>, fine_line(m) * sizeof(lcx<double>)};
         MM_XLANE_SHAPES(MM_CASE)
 #undef MM_CASE
