@@ -22,6 +22,7 @@ struct ClassHost {
     int* d_members = nullptr;
     void* S = nullptr;             // spectra [member][3][PyA][Wk] complex
     float* Hd = nullptr;           // demag field [member][3][ny][nx]
+    float* noise = nullptr;        // thermal field of a step, same layout (null: drawn in both stages)
 };
 
 struct BatchHost {
@@ -88,6 +89,7 @@ void batch_free(BatchHost* b) {
         cudaFree(k.d_members);
         cudaFree(k.S);
         cudaFree(k.Hd);
+        cudaFree(k.noise);
     }
     for (auto& p : b->plans) demag_free_plan(p);
     delete b;
@@ -438,8 +440,11 @@ static void stacked_stage(mm_ctx* c, BatchHost* b, int stage) {
         a.ms = (float*)c->d_mtmp;
         a.k1 = (float*)c->d_k[0];
         a.hd = demag ? k.Hd : nullptr;
+        a.noise = k.noise;
         batch_field_args(c, a.fa);
         a.fa.terms = c->terms;
+        a.fa.R0 = c->r0f;
+        a.fa.c_uniform = c->c00f;
         a.stage = stage;
         a.dm = c->integrator == MM_DM ? 1 : 0;
         a.ext = c->ext_terms ? 1 : 0;
@@ -500,6 +505,13 @@ void batch_set_shape(BatchHost* b, int nt, int blocks) {
             }
         }
         if (ok) {
+            for (ClassHost& k : b->ch) {
+                const size_t nb = sizeof(float) * (size_t)k.Rc * 3 * k.nx * k.ny;
+                if (!k.noise && cudaMalloc(&k.noise, nb) != cudaSuccess) {
+                    k.noise = nullptr;
+                    cudaGetLastError();
+                }
+            }
             b->stacked = true;
             return;
         }

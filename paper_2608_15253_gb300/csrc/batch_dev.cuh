@@ -453,6 +453,7 @@ struct StackArgs {
     float* ms;              // predictor state
     float* k1;              // predictor slope / rotation vector
     const float* hd;        // the class's demag field [member][3][ny][nx], or null
+    float* noise;           // its thermal field of the step, drawn by stage 1 for stage 2, or null
     FieldArgs<float> fa;
     int stage;              // 1 predictor, 2 corrector
     int dm;

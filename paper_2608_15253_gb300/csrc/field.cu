@@ -287,6 +287,10 @@ constexpr size_t c2r_field_smem(int rpc) {
     return lines > rows ? lines : rows;
 }
 
+// cells per thread: four in the short QUIET form; two otherwise (half the code
+// and twice the threads: instruction fetches and latency bound those launches)
+template <bool QUIET> constexpr int c2r_v() { return QUIET ? 4 : 2; }
+
 template <int M, int G, int Q, bool EXT, bool QUIET = false>
 __global__ void __launch_bounds__(kC2RThreads, QUIET ? 2 : 1) c2r_field_kernel(FieldArgs<float> a, C2RSpec s) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -309,13 +313,14 @@ __global__ void __launch_bounds__(kC2RThreads, QUIET ? 2 : 1) c2r_field_kernel(F
         __syncthreads();
     }
     __syncthreads();
-    const int tpr = nx / 4;
+    constexpr int V = c2r_v<QUIET>();
+    const int tpr = nx / V;
     for (int c = threadIdx.x; c < rpc * tpr; c += blockDim.x) {
-        const int rl = c / tpr, x0 = 4 * (c - rl * tpr);
+        const int rl = c / tpr, x0 = V * (c - rl * tpr);
         const int row = row0 + rl;
         if (row < nrows) {
             const int z = row / a.ny, y = row - z * a.ny;
-            field_vec_cells<4, EXT, true, QUIET>(a, x0, y, z, sH + rl * 3 * nx + x0, nx);
+            field_vec_cells<V, EXT, true, QUIET>(a, x0, y, z, sH + rl * 3 * nx + x0, nx);
         }
     }
     if (!QUIET && a.tick) fixed_finish(const_cast<DevState*>(a.st), a.tick);
@@ -350,6 +355,8 @@ static FieldArgs<T> field_args(mm_ctx* c, int mode, unsigned terms, const T* m, 
     a.key1 = (uint32_t)(c->seed >> 32);
     const double V = g.dx * g.dy * g.dz;
     a.th_scale = c->Tr > 0 ? (T)std::sqrt(c->Tr / (V * c->cfg.dt)) : (T)0;
+    // the predictor's draw serves the corrector (one draw per step by the scheme)
+    a.noise = mode == MODE_HEUN1 || mode == MODE_HEUN2 || mode == MODE_DM1 || mode == MODE_DM2 ? (T*)c->d_hbuf : nullptr;
     a.st = c->d_state;
     a.step_override = step_override;
     a.cubic_w1 = c->cubic_energy ? (T)0.5 : (T)1;
@@ -510,7 +517,7 @@ void field_c2r_launch(mm_ctx* c, int mode, unsigned terms, const void* m, void* 
         const int rpc = c2r_rows(G_, rows);                                                                   \
         const C2RSpec sp{(const float2*)d.spec, (const float2*)d.tw_x, d.PyA, d.Wk, rpc};                     \
         const unsigned grid = (unsigned)((rows + rpc - 1) / rpc);                                             \
-        const int fft = (3 * rpc * G_ + 31) / 32 * 32, cells = (rpc * c->grid.nx / 4 + 31) / 32 * 32;         \
+        const int fft = (3 * rpc * G_ + 31) / 32 * 32, cells = (rpc * c->grid.nx / (quiet ? 4 : 2) + 31) / 32 * 32; \
         const int nt = std::max(fft, std::min(kC2RThreads, cells));                                           \
         const size_t smem = c2r_field_smem<M_, G_, Q_>(rpc);                                                  \
         if (c->ext_terms) launch_dep(c2r_field_kernel<M_, G_, Q_, true>, grid, nt, smem, c, a, sp);           \

@@ -76,6 +76,7 @@ struct FieldArgs {
     // thermal
     uint32_t key0, key1;
     T th_scale;           // sqrt(T / (V dt)); sigma = lut.sigma0 * th_scale
+    T* noise;             // [3][N]: the step's thermal field, kept by the predictor for the corrector, or null
     const DevState* st;   // step counter, dt, active flag
     int gate;             // 1: skip the launch when st->active == 0
     long long step_override;  // >= 0: use this step for the noise
@@ -239,7 +240,15 @@ __device__ __forceinline__ void cell_field_nb(const FieldArgs<T>& a, long long i
         if (use_hd) H = H + hdv;
         else if (a.Hd) H = H + ld3(a.Hd, N, i);
     }
-    if (!QUIET && (a.terms & MM_TERM_THERMAL) && a.th_scale != (T)0) H = H + thermal_h<T>(a, i, R, step);
+    if (!QUIET && (a.terms & MM_TERM_THERMAL) && a.th_scale != (T)0) {
+        if (a.noise && (a.mode == MODE_HEUN2 || a.mode == MODE_DM2)) {
+            H = H + ld3(a.noise, N, i);
+        } else {
+            const v3<T> th = thermal_h<T>(a, i, R, step);
+            if (a.noise) st3(a.noise, N, i, th);
+            H = H + th;
+        }
+    }
     if (!want_k) return;
     // LLG torque, Eq. 1: -gamma' mu0 [m x H + alpha m x (m x H)]
     const v3<T> mxH = cross(m, H);
