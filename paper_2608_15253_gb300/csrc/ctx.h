@@ -229,7 +229,7 @@ void thermal_raw_launch(mm_ctx* c, long long step, uint32_t* d_raw, void* d_h);
 // inverse X pass + field kernel in one launch (the demag spectrum of the
 // state must be ready); field_c2r_fusable says whether the grid allows it
 bool field_c2r_fusable(const mm_ctx* c);
-cudaError_t field_c2r_setup();
+cudaError_t field_c2r_setup(const mm_ctx* c);
 void field_c2r_launch(mm_ctx* c, int mode, unsigned terms, const void* m, void* out, void* out2, const void* m0,
                       const void* k1, long long step_override, int gate, int kstage, bool finish = false);
 

@@ -1107,6 +1107,8 @@ static mm_status demag_setup_t(mm_ctx* c) {
     cudaFree(sp);
     free_tw64();
     if (e != cudaSuccess) return cuda_check(c, e, "demag setup");
+    if (sizeof(T) == 4) e = field_c2r_setup(c);
+    if (e != cudaSuccess) return cuda_check(c, e, "field kernel attributes");
     d.on = 1;
     return MM_OK;
 }
@@ -1140,7 +1142,6 @@ mm_status demag_setup(mm_ctx* c) {
         tw32[q] = make_float2((float)std::cos(ang), (float)std::sin(ang));
     }
     cudaError_t e = cudaMemcpyToSymbol(c_tw32, tw32, sizeof tw32);
-    if (e == cudaSuccess) e = field_c2r_setup();
     if (e != cudaSuccess) return cuda_check(c, e, "twiddle table");
     e = fft_attributes<float>();
     if (e == cudaSuccess) e = fft_attributes<double>();

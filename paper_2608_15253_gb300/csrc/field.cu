@@ -14,79 +14,10 @@
 
 #include "common.cuh"
 #include "ctx.h"
-#include "field_dev.cuh"
+#include "field_x.cuh"
 #include "launch.h"
-#include "lane_x.cuh"
 
 namespace mm {
-
-// Output of one present cell for the launch's mode: H, the slope k (to
-// `out` or to the FSAL slot of stage kstage), the Heun / Depondt-Mertens
-// predictor (m*, with k or Omega to out2) or corrector (renormalised); the
-// step is the attempt's dt_eff (the fixed dt for the fixed-step schemes).
-template <typename T>
-__device__ __forceinline__ void cell_store(const FieldArgs<T>& a, long long i, const v3<T>& m, const v3<T>& H,
-                                           const v3<T>& k) {
-    const long long N = a.N;
-    if (a.mode == MODE_H) {
-        st3(a.out, N, i, H);
-    } else if (a.mode == MODE_K) {
-        T* o = a.out;
-        if (!o) {
-            const int kf = a.st->k_first;
-            o = a.kptr[a.kstage == 0 ? kf : 6 - kf];
-        }
-        st3(o, N, i, k);
-    } else if (a.mode == MODE_HEUN1) {
-        const T dt = (T)a.st->dt_eff;
-        st3(a.out2, N, i, k);
-        st3(a.out, N, i, m + dt * k);
-    } else if (a.mode == MODE_HEUN2) {  // m_new = normalise(m0 + dt/2 (k1 + k2))
-        const T dt = (T)a.st->dt_eff;
-        const v3<T> m0 = ld3(a.m0, N, i);
-        const v3<T> k1 = ld3(a.k1, N, i);
-        v3<T> mn = m0 + ((T)0.5 * dt) * (k1 + k);
-        const T inv = (T)1 / sqrt(dot(mn, mn));
-        st3(a.out, N, i, inv * mn);
-    } else if (a.mode == MODE_DM1) {   // Omega_1 and m* = R(Omega_1 dt) m
-        const T dt = (T)a.st->dt_eff;
-        st3(a.out2, N, i, k);
-        st3(a.out, N, i, rodrigues<T>(m, k, dt));
-    } else {  // MODE_DM2: m_new = R((Omega_1 + Omega_2) dt / 2) m0
-        const T dt = (T)a.st->dt_eff;
-        const v3<T> m0 = ld3(a.m0, N, i);
-        const v3<T> w1 = ld3(a.k1, N, i);
-        const v3<T> mn = rodrigues<T>(m0, (T)0.5 * (w1 + k), dt);
-        const T inv = (T)1 / sqrt(dot(mn, mn));
-        st3(a.out, N, i, inv * mn);
-    }
-}
-
-// UNIF: one material (coefficients passed by value in the launch
-// parameters, no region map or coefficient-table loads).
-template <typename T, bool UNIF, bool EXT>
-__device__ __forceinline__ void field_cell(const FieldArgs<T>& a, int x, int y, int z) {
-    const long long N = a.N;
-    const long long i = ((long long)z * a.ny + y) * a.nx + x;
-    const int ri = UNIF ? 0 : (a.region ? a.region[i] : 0);
-    const Region<T>& R = UNIF ? a.R0 : a.lut[ri];
-    const v3<T> m = ld3(a.m, N, i);
-    if (R.present == (T)0) {
-        const v3<T> zero = mk3<T>(0, 0, 0);
-        T* o = a.out;
-        if (!o) {
-            const int kf = a.st->k_first;
-            o = a.kptr[a.kstage == 0 ? kf : 6 - kf];
-        }
-        if (a.mode == MODE_HEUN1 || a.mode == MODE_DM1) { st3(o, N, i, zero); st3(a.out2, N, i, zero); }
-        else st3(o, N, i, zero);
-        return;
-    }
-    const long long step = a.step_override >= 0 ? a.step_override : (a.st ? a.st->step : 0);
-    v3<T> H, k;
-    cell_field<T, UNIF, EXT>(a, x, y, z, i, ri, R, m, nullptr, step, H, k, a.mode != MODE_H, a.mode >= MODE_DM1);
-    cell_store<T>(a, i, m, H, k);
-}
 
 template <typename T, bool UNIF, bool EXT>
 __global__ void __launch_bounds__(256) field_kernel(FieldArgs<T> a) {
@@ -98,163 +29,6 @@ __global__ void __launch_bounds__(256) field_kernel(FieldArgs<T> a) {
     if (a.tick) fixed_finish(const_cast<DevState*>(a.st), a.tick);
 }
 
-// One material, FP32, nx a multiple of V (2 or 4): each thread owns V
-// consecutive cells of a row.  The state, its y/z neighbours, the demag
-// field and the outputs move as 8- or 16-byte vectors; the x neighbours of
-// the inner cells come from the thread's own registers, only the two
-// row-end neighbours are scalar loads.
-template <int V> struct fvec;
-template <> struct fvec<2> { using t = float2; };
-template <> struct fvec<4> { using t = float4; };
-
-template <int V>
-__device__ __forceinline__ typename fvec<V>::t ldv(const float* p) {
-    return __ldg(reinterpret_cast<const typename fvec<V>::t*>(p));
-}
-template <int V>
-__device__ __forceinline__ void stv(float* p, const typename fvec<V>::t& v) {
-    *reinterpret_cast<typename fvec<V>::t*>(p) = v;
-}
-__device__ __forceinline__ float fget(const float2& v, int q) { return q == 0 ? v.x : v.y; }
-__device__ __forceinline__ float fget(const float4& v, int q) { return q == 0 ? v.x : q == 1 ? v.y : q == 2 ? v.z : v.w; }
-__device__ __forceinline__ void fset(float2& v, int q, float x) { if (q == 0) v.x = x; else v.y = x; }
-__device__ __forceinline__ void fset(float4& v, int q, float x) {
-    if (q == 0) v.x = x; else if (q == 1) v.y = x; else if (q == 2) v.z = x; else v.w = x;
-}
-
-// The V cells x0 .. x0 + V - 1 of row (z, y).  HD_SMEM: the demag field of
-// the cells comes from shared memory (hds[c * hd_stride + q], the fused
-// inverse-X-pass kernel below), else from a.Hd in global memory.  QUIET:
-// slopes only (MODE_K), no thermal field, no spin torque -- the variant for
-// deterministic runs without current, with far fewer registers.
-template <int V, bool EXT, bool HD_SMEM, bool QUIET = false>
-__device__ __forceinline__ void field_vec_cells(const FieldArgs<float>& a, int x0, int y, int z, const float* hds,
-                                                int hd_stride) {
-    using VT = typename fvec<V>::t;
-    const long long N = a.N;
-    const long long i0 = ((long long)z * a.ny + y) * a.nx + x0;
-    const Region<float>& R = a.R0;
-    const long long step = a.step_override >= 0 ? a.step_override : (a.st ? a.st->step : 0);
-    VT mc[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) mc[c] = ldv<V>(a.m + c * N + i0);
-    const unsigned nbt = MM_TERM_EXCHANGE | MM_TERM_DMI | (EXT ? MM_TERM_SURFACE : 0u);
-    const bool need_nb = (a.terms & nbt) || (!QUIET && a.tq == MM_TORQUE_ZL);
-    // neighbour rows (y+, y-, z+, z-) as vectors, row-end x neighbours as scalars
-    VT nr[4][3];
-    bool rin[4] = {false, false, false, false};
-    float xl[3] = {0, 0, 0}, xr[3] = {0, 0, 0};
-    bool lin = false, rinx = false;
-    if (need_nb) {
-        const long long sy = a.nx, sz = (long long)a.nx * a.ny;
-        const int ny = a.ny, nz = a.nz;
-        const int qs[4] = {y + 1, y - 1, z + 1, z - 1};
-        const int dm[4] = {ny, ny, nz, nz};
-        const int pr[4] = {a.py, a.py, a.pz, a.pz};
-        const int ps[4] = {y, y, z, z};
-        const long long st[4] = {sy, sy, sz, sz};
-#pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            int q = qs[s];
-            bool inside = q >= 0 && q < dm[s];
-            if (!inside && pr[s]) { q = (q + dm[s]) % dm[s]; inside = true; }
-            rin[s] = inside;
-            if (inside) {
-                const long long j = i0 + (long long)(q - ps[s]) * st[s];
-#pragma unroll
-                for (int c = 0; c < 3; ++c) nr[s][c] = ldv<V>(a.m + c * N + j);
-            }
-        }
-        int ql = x0 - 1, qr = x0 + V;
-        lin = ql >= 0;
-        rinx = qr < a.nx;
-        if (!lin && a.px) { ql += a.nx; lin = true; }
-        if (!rinx && a.px) { qr -= a.nx; rinx = true; }
-        const long long row = i0 - x0;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            if (lin) xl[c] = __ldg(a.m + c * N + row + ql);
-            if (rinx) xr[c] = __ldg(a.m + c * N + row + qr);
-        }
-    }
-    VT hd[3];
-    const bool dem = (a.terms & MM_TERM_DEMAG) && (HD_SMEM || a.Hd);
-    if (dem) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-            hd[c] = HD_SMEM ? *reinterpret_cast<const VT*>(hds + c * hd_stride) : ldv<V>(a.Hd + c * N + i0);
-    }
-    VT o1[3], o2[3];
-#pragma unroll
-    for (int q = 0; q < V; ++q) {
-        const v3<float> m = mk3<float>(fget(mc[0], q), fget(mc[1], q), fget(mc[2], q));
-        v3<float> nbv[6];
-        bool nbp[6];
-        float cnb[6];
-        if (need_nb) {
-            // x+ / x-
-            const bool pp = q < V - 1 || rinx, pm = q > 0 || lin;
-            nbp[0] = pp;
-            nbp[1] = pm;
-            nbv[0] = q < V - 1 ? mk3<float>(fget(mc[0], q + 1), fget(mc[1], q + 1), fget(mc[2], q + 1))
-                               : (rinx ? mk3<float>(xr[0], xr[1], xr[2]) : ghost_value<float, EXT>(m, 0, 1, a.hx, R.ratio, R.ratio_b));
-            nbv[1] = q > 0 ? mk3<float>(fget(mc[0], q - 1), fget(mc[1], q - 1), fget(mc[2], q - 1))
-                           : (lin ? mk3<float>(xl[0], xl[1], xl[2]) : ghost_value<float, EXT>(m, 0, -1, a.hx, R.ratio, R.ratio_b));
-            cnb[0] = pp ? a.c_uniform : R.cg;
-            cnb[1] = pm ? a.c_uniform : R.cg;
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                const int slot = 2 + s, d = 1 + s / 2, sg = (s & 1) ? -1 : 1;
-                nbp[slot] = rin[s];
-                nbv[slot] = rin[s] ? mk3<float>(fget(nr[s][0], q), fget(nr[s][1], q), fget(nr[s][2], q))
-                                   : ghost_value<float, EXT>(m, d, sg, d == 1 ? a.hy : a.hz, R.ratio, R.ratio_b);
-                cnb[slot] = rin[s] ? a.c_uniform : R.cg;
-            }
-        }
-        const v3<float> hq = dem ? mk3<float>(fget(hd[0], q), fget(hd[1], q), fget(hd[2], q)) : mk3<float>(0, 0, 0);
-        v3<float> H, k;
-        cell_field_nb<float, EXT, QUIET>(a, i0 + q, R, m, nbv, nbp, cnb, dem, hq, step, H, k,
-                                         QUIET || a.mode != MODE_H, !QUIET && a.mode >= MODE_DM1);
-        v3<float> r1 = H, r2 = k;
-        if (QUIET || a.mode == MODE_K) r1 = k;
-        else if (QUIET) {
-        } else if (a.mode == MODE_HEUN1) {
-            const float dt = (float)a.st->dt_eff;
-            r1 = m + dt * k;
-            r2 = k;
-        } else if (a.mode == MODE_HEUN2) {
-            const float dt = (float)a.st->dt_eff;
-            const long long i = i0 + q;
-            const v3<float> m0 = ld3(a.m0, N, i);
-            const v3<float> k1 = ld3(a.k1, N, i);
-            v3<float> mn = m0 + (0.5f * dt) * (k1 + k);
-            r1 = (1.0f / sqrtf(dot(mn, mn))) * mn;
-        } else if (a.mode == MODE_DM1) {
-            r1 = rodrigues<float>(m, k, (float)a.st->dt_eff);
-            r2 = k;
-        } else if (a.mode == MODE_DM2) {
-            const long long i = i0 + q;
-            const v3<float> m0 = ld3(a.m0, N, i);
-            const v3<float> w1 = ld3(a.k1, N, i);
-            const v3<float> mn = rodrigues<float>(m0, 0.5f * (w1 + k), (float)a.st->dt_eff);
-            r1 = (1.0f / sqrtf(dot(mn, mn))) * mn;
-        }
-        fset(o1[0], q, r1.x); fset(o1[1], q, r1.y); fset(o1[2], q, r1.z);
-        fset(o2[0], q, r2.x); fset(o2[1], q, r2.y); fset(o2[2], q, r2.z);
-    }
-    float* o = a.out;
-    if (!o) {
-        const int kf = a.st->k_first;
-        o = a.kptr[a.kstage == 0 ? kf : 6 - kf];
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) stv<V>(o + c * N + i0, o1[c]);
-    if (!QUIET && (a.mode == MODE_HEUN1 || a.mode == MODE_DM1)) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) stv<V>(a.out2 + c * N + i0, o2[c]);
-    }
-}
-
 template <int V, bool EXT, bool QUIET = false>
 __global__ void __launch_bounds__(256) field_vec_kernel(FieldArgs<float> a) {
     dep_wait();
@@ -262,67 +36,6 @@ __global__ void __launch_bounds__(256) field_vec_kernel(FieldArgs<float> a) {
     const int x0 = V * (blockIdx.x * blockDim.x + threadIdx.x);
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x0 < a.nx && y < a.ny) field_vec_cells<V, EXT, false, QUIET>(a, x0, y, blockIdx.z, nullptr, 0);
-    if (!QUIET && a.tick) fixed_finish(const_cast<DevState*>(a.st), a.tick);
-}
-
-// The last demag pass (inverse X, half spectrum -> real rows) fused with
-// the field kernel: the first 3 G rows_per_cta threads of a CTA run the C2R of
-// the three components of its rows (z, y), G threads each (lane_x.cuh), into
-// shared memory over the exchange buffers; then every thread forms the field,
-// torque and stage output of 4 cells at a time with the demag field read from
-// there -- H_demag never goes through global memory.
-struct C2RSpec {
-    const float2* spec;     // [3][nz][PyA][Wk]
-    const float2* tw;       // exp(-2 pi i q / Px)
-    int PyA, Wk;
-    int rpc;                // rows per CTA
-};
-
-constexpr int kC2RThreads = 192;
-// exchange lines of the C2R threads in whole warps, and the field rows over them
-template <int M, int G, int Q>
-constexpr size_t c2r_field_smem(int rpc) {
-    const size_t tasks = (3 * rpc * G + 31) / 32 * 32 / G;
-    const size_t lines = tasks * XSplit<M, G, Q>::LINE * sizeof(float2), rows = (size_t)3 * rpc * M * sizeof(float);
-    return lines > rows ? lines : rows;
-}
-
-// cells per thread: four in the short QUIET form; two otherwise (half the code
-// and twice the threads: instruction fetches and latency bound those launches)
-template <bool QUIET> constexpr int c2r_v() { return QUIET ? 4 : 2; }
-
-template <int M, int G, int Q, bool EXT, bool QUIET = false>
-__global__ void __launch_bounds__(kC2RThreads, QUIET ? 2 : 1) c2r_field_kernel(FieldArgs<float> a, C2RSpec s) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    dep_wait();
-    if (a.gate && !a.st->active) return;
-    float* sH = reinterpret_cast<float*>(smem_raw);   // [rpc][3][nx], once the lines are in registers
-    const int nx = a.nx, rpc = s.rpc, nrows = a.ny * a.nz;
-    const int row0 = blockIdx.x * rpc;
-    if ((int)threadIdx.x < (3 * rpc * G + 31) / 32 * 32) {
-        const int task = threadIdx.x / G, rl = task / 3, comp = task - 3 * rl, row = row0 + rl;
-        const bool valid = rl < rpc && row < nrows;
-        const int z = valid ? row / a.ny : 0, y = valid ? row - z * a.ny : 0;
-        const float2* X = s.spec + ((long long)(comp * a.nz + z) * s.PyA + y) * s.Wk;
-        lcx<float>* line = reinterpret_cast<lcx<float>*>(smem_raw) + task * XSplit<M, G, Q>::LINE;
-        float* dst = sH + (rl * 3 + comp) * nx;
-        lane_c2r_row<float, M, G, Q>(X, s.tw, line, threadIdx.x % G, valid, [] { __syncthreads(); }, [&](int n, float2 v) {
-            if (valid && 2 * n < nx) *reinterpret_cast<float2*>(dst + 2 * n) = v;
-        });
-    } else {
-        __syncthreads();
-    }
-    __syncthreads();
-    constexpr int V = c2r_v<QUIET>();
-    const int tpr = nx / V;
-    for (int c = threadIdx.x; c < rpc * tpr; c += blockDim.x) {
-        const int rl = c / tpr, x0 = V * (c - rl * tpr);
-        const int row = row0 + rl;
-        if (row < nrows) {
-            const int z = row / a.ny, y = row - z * a.ny;
-            field_vec_cells<V, EXT, true, QUIET>(a, x0, y, z, sH + rl * 3 * nx + x0, nx);
-        }
-    }
     if (!QUIET && a.tick) fixed_finish(const_cast<DevState*>(a.st), a.tick);
 }
 
@@ -457,47 +170,38 @@ void field_launch(mm_ctx* c, int mode, unsigned terms, const void* m, const void
                                (const double*)m0, (const double*)k1, step_override, gate, kstage, finish);
 }
 
-// Inverse X pass + field kernel in one launch (FP32, one material, nx a
-// multiple of 4 dividing 1024 and equal to the half length).  One GB300:
-// 512x512x64 293 us (307 with a row per warp and three transforms in turn),
-// 256x256x16 26.6 (27.9), a 512x512 film 12.8 (16.7), a 256x256 film at 300 K
-// with spin-orbit torque 14.8 (19.9).  The two separate kernels take 198 + 201
-// us at 512x512x64.
-#define MM_C2R_FIELD_LENGTHS(X) X(128, 8, 16) X(256, 8, 32) X(512, 16, 32)
-
+// Inverse X pass + field kernel in one launch (FP32, one material, even nx,
+// any length of the X passes' register kernels).  One GB300, against the two
+// kernels: 512x512x64 256 us (198 + 201), 250x250x40 56 us (35 + 55),
+// 256x256x16 26.3 us, a 200x50 film 8.7 us (8.1 + 9.4).  Region maps and odd rows
+// take the two kernels: a cell at a time in this one, 150x150x24 with a region
+// map took 44 us against 11.3 + 21.
 bool field_c2r_fusable(const mm_ctx* c) {
     const mm_grid& g = c->grid;
     if (c->prec != 32 || !c->dm.on || !c->uniform || c->d_region || c->r0f.present == 0.f) return false;
-    if (g.nx % 4 != 0 || 1024 % g.nx != 0 || c->dm.Lh != g.nx) return false;
-    switch (c->dm.Lh) {
-#define MM_CASE(m, g, q) case m: return true;
-        MM_C2R_FIELD_LENGTHS(MM_CASE)
-#undef MM_CASE
-        default: return false;
-    }
+    return g.nx % 2 == 0 && g.nx <= c->dm.Lh && field_x_full(c->dm.Lh).group > 0;
 }
 
-// rows per CTA: as many as kC2RThreads threads transform at once, fewer on
-// small grids so that two CTAs per SM run
-static int c2r_rows(int G, long long rows) {
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+// rows per CTA: as many as 96 threads transform at once (at least one; 192
+// threads at 12 warps an SM were slower, see the kernel), fewer on small grids
+// so that two CTAs per SM run
+static int c2r_rows(int G, long long rows, int sms) {
     const long long want = (rows + 2 * sms - 1) / (2 * sms);
-    return (int)std::max(1LL, std::min<long long>(kC2RThreads / (3 * G), want));
+    return (int)std::max(1LL, std::min<long long>(96 / (3 * G), want));
 }
 
-cudaError_t field_c2r_setup() {
+// opts the kernels of the plan's length into their shared memory and loads
+// them, outside any stream capture
+cudaError_t field_c2r_setup(const mm_ctx* c) {
     cudaError_t e = cudaSuccess;
-    const auto opt = [&](const void* k, size_t smem) {
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    };
-#define MM_CASE(m, g, q)                                                                                      \
-    opt((const void*)c2r_field_kernel<m, g, q, true>, c2r_field_smem<m, g, q>(kC2RThreads / (3 * g)));          \
-    opt((const void*)c2r_field_kernel<m, g, q, false>, c2r_field_smem<m, g, q>(kC2RThreads / (3 * g)));         \
-    opt((const void*)c2r_field_kernel<m, g, q, false, true>, c2r_field_smem<m, g, q>(kC2RThreads / (3 * g)));
-    MM_C2R_FIELD_LENGTHS(MM_CASE)
-#undef MM_CASE
+    if (c->prec != 32) return e;
+    const int M = c->dm.Lh;
+    for (const FieldX& f : {field_x_quiet(M), field_x_full(M), field_x_ext(M)}) {
+        if (f.group == 0) continue;
+        const size_t smem = field_x_smem(f.group, f.line, M, std::max(1, 96 / (3 * f.group)));
+        for (const auto kern : f.kern)
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    }
     return e;
 }
 
@@ -507,28 +211,23 @@ void field_c2r_launch(mm_ctx* c, int mode, unsigned terms, const void* m, void* 
                                            (const float*)m0, (const float*)k1, step_override, gate, kstage);
     if (finish) a.tick = c->d_tick;
     const DemagPlan& d = c->dm;
+    const int nx = c->grid.nx;
     const long long rows = (long long)c->grid.ny * c->grid.nz;
-    const double bytes = field_bytes(c, mode, terms, false) + 3.0 * rows * (d.Kx * sizeof(float2));
-    LaunchScope ls(c, "c2r_field", bytes);
-    const bool quiet = field_quiet(c, mode, terms, a);
-    switch (d.Lh) {
-#define MM_CASE(M_, G_, Q_)                                                                                   \
-    case M_: {                                                                                                \
-        const int rpc = c2r_rows(G_, rows);                                                                   \
-        const C2RSpec sp{(const float2*)d.spec, (const float2*)d.tw_x, d.PyA, d.Wk, rpc};                     \
-        const unsigned grid = (unsigned)((rows + rpc - 1) / rpc);                                             \
-        const int fft = (3 * rpc * G_ + 31) / 32 * 32, cells = (rpc * c->grid.nx / (quiet ? 4 : 2) + 31) / 32 * 32; \
-        const int nt = std::max(fft, std::min(kC2RThreads, cells));                                           \
-        const size_t smem = c2r_field_smem<M_, G_, Q_>(rpc);                                                  \
-        if (c->ext_terms) launch_dep(c2r_field_kernel<M_, G_, Q_, true>, grid, nt, smem, c, a, sp);           \
-        else if (quiet) launch_dep(c2r_field_kernel<M_, G_, Q_, false, true>, grid, nt, smem, c, a, sp);      \
-        else launch_dep(c2r_field_kernel<M_, G_, Q_, false>, grid, nt, smem, c, a, sp);                       \
-        break;                                                                                                \
-    }
-        MM_C2R_FIELD_LENGTHS(MM_CASE)
-#undef MM_CASE
-        default: break;
-    }
+    const bool quiet = !c->ext_terms && field_quiet(c, mode, terms, a);
+    const FieldX f = c->ext_terms ? field_x_ext(d.Lh) : quiet ? field_x_quiet(d.Lh) : field_x_full(d.Lh);
+    const int four = quiet && nx % 4 == 0;
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int rpc = c2r_rows(f.group, rows, sms);
+    const long long grid = (rows + rpc - 1) / rpc;
+    const C2RSpec sp{(const float2*)d.spec, (const float2*)d.tw_x, d.PyA, d.Wk, rpc};
+    // grids that fill the chip with CTAs of 96 threads: five of them per SM; on
+    // smaller ones more threads share the cells (a 512x512 film: 12.0 us against 14.2)
+    const int cells = (rpc * nx / (four ? 4 : 2) + 31) / 32 * 32, most = grid >= 5LL * sms ? 96 : kC2RThreads;
+    LaunchScope ls(c, "c2r_field", field_bytes(c, mode, terms, false) + 3.0 * rows * (d.Kx * sizeof(float2)));
+    launch_dep(f.kern[four], (unsigned)grid, std::max(field_x_fft(f.group, rpc), std::min(most, cells)),
+               field_x_smem(f.group, f.line, nx, rpc), c, a, sp);
 }
 
 // Raw Philox words and the thermal field of every cell at a given step.

@@ -134,6 +134,37 @@ def test_stage_state_formed_in_the_x_pass(shape, prec):
         mm.mm_destroy(ctx)
 
 
+@pytest.mark.parametrize("kind", ["slopes", "current", "cubic"])
+@pytest.mark.parametrize("L", X_LENGTHS)
+def test_x_pass_inside_the_field_kernel(L, kind):
+    """FP32 rows padded to L, of the smallest and the largest even length (four
+    cells a thread where four divide it): two RK4 steps, two Heun steps with a
+    current and a temperature, two RK4 steps with the further local terms,
+    against the FP64 oracle."""
+    mm = need_gpu()
+    from oracle.llg import Solver, Torque, replica_seed
+    below = max([v for v in LENGTHS if v % 2 == 0 and v < L])
+    lo = below // 2 + 1
+    for nx in sorted({lo + lo % 2, L // 2 - L // 2 % 2}):
+        grid = W.Grid(nx, 5, 2, 2e-9, 2e-9, 2e-9)
+        mat = W.Material(Ms=8.0e5, A=1.3e-11, alpha=0.02, Kc1=4.5e4 if kind == "cubic" else 0.0)
+        terms = ("exchange", "zeeman", "demag") + (("cubic",) if kind == "cubic" else ())
+        m0 = W.m_perp(grid, seed=nx, tilt=0.3)
+        T, tq = (300.0, Torque(kind="sot", J=2e11, p=(0, 1, 0), theta_SH=0.1, fl_ratio=0.3)) if kind == "current" else (0.0, Torque())
+        o = Solver(oracle_problem(grid, mat), m0, terms=terms, dt=1e-14, T=T, seed=replica_seed(5, 0), torque=tq)
+        ctx = make_ctx(mm, grid, mat, precision=32, dt=1e-14, T=T, seed=5, integrator="heun" if T else "rk4")
+        try:
+            if T:
+                mm.mm_set_torque(ctx, mm.make_torque(mm.MM_TORQUE_SOT, p=(0, 1, 0), theta_SH=0.1, fl_ratio=0.3), 2e11)
+            mm.mm_set_m(ctx, 0, m0)
+            mm.mm_step(ctx, 2)
+            for _ in range(2):
+                o.heun_step() if T else o.rk4_step()
+            assert np.abs(mm.mm_get_m(ctx, 0, m0.shape) - o.m).max() <= 1e-5, nx
+        finally:
+            mm.mm_destroy(ctx)
+
+
 @pytest.mark.parametrize("integrator", ["heun", "dm"])
 @pytest.mark.parametrize("n", [(8, 8), (7, 8), (12, 12), (16, 16), (15, 16), (16, 15), (24, 24), (32, 32), (31, 32)])
 def test_small_film_ensembles_match_oracle(n, integrator):
