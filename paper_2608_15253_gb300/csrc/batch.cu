@@ -430,7 +430,6 @@ static void stacked_stage(mm_ctx* c, BatchHost* b, int stage) {
     for (size_t q = 0; q < b->ch.size(); ++q) {
         ClassHost& k = b->ch[q];
         const float* in = (const float*)(stage == 1 ? c->d_m : c->d_mtmp) + k.off0;
-        if (demag) demag_apply_stacked2d(c, b->plans[q], in, k.Hd, k.S, k.nx, k.ny, k.Rc);
         StackArgs a{};
         a.rep = b->d_rep;
         a.members = k.d_members;
@@ -439,7 +438,6 @@ static void stacked_stage(mm_ctx* c, BatchHost* b, int stage) {
         a.m0 = (float*)c->d_m;
         a.ms = (float*)c->d_mtmp;
         a.k1 = (float*)c->d_k[0];
-        a.hd = demag ? k.Hd : nullptr;
         a.noise = k.noise;
         batch_field_args(c, a.fa);
         a.fa.terms = c->terms;
@@ -449,10 +447,14 @@ static void stacked_stage(mm_ctx* c, BatchHost* b, int stage) {
         a.dm = c->integrator == MM_DM ? 1 : 0;
         a.ext = c->ext_terms ? 1 : 0;
         a.st = c->d_state;
+        const bool fused = demag && stacked_x_fusable(a, b->plans[q].Lh);
+        a.hd = demag && !fused ? k.Hd : nullptr;
+        if (demag) demag_apply_stacked2d(c, b->plans[q], in, fused ? nullptr : k.Hd, k.S, k.nx, k.ny, k.Rc);
         const double cells = (double)k.Rc * k.nx * k.ny;
         LaunchScope ls(c, stage == 1 ? "stacked_field1" : "stacked_field2",
                        cells * (stage == 1 ? 36.0 : 48.0) + (demag ? cells * 12.0 : 0.0));
-        stacked_field_launch(a, k.Rc, c->stream);
+        if (fused) stacked_x_launch(a, k.Rc, b->plans[q], k.S, c->stream);
+        else stacked_field_launch(a, k.Rc, c->stream);
     }
 }
 
@@ -489,7 +491,9 @@ void batch_set_shape(BatchHost* b, int nt, int blocks) {
         for (size_t q = 0; q < b->ch.size() && ok; ++q) {
             ClassHost& k = b->ch[q];
             const DemagPlan& p = b->plans[q];
-            if (!p.on || (k.S && k.Hd)) continue;
+            if (!p.on) continue;
+            ok = stacked_x_setup(p.Lh) == cudaSuccess;
+            if (!ok || (k.S && k.Hd)) continue;
             cudaFree(k.S);
             cudaFree(k.Hd);
             k.S = nullptr;

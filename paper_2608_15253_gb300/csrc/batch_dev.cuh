@@ -461,6 +461,10 @@ struct StackArgs {
     const DevState* st;
 };
 void stacked_field_launch(const StackArgs& a, int Rc, cudaStream_t s);
+// the same with the inverse X pass of the class's spectra S inside
+bool stacked_x_fusable(const StackArgs& a, int Lh);
+cudaError_t stacked_x_setup(int Lh);
+void stacked_x_launch(const StackArgs& a, int Rc, const DemagPlan& p, const void* S, cudaStream_t s);
 void stacked_trials_launch(const BatchArgs& a, int R, cudaStream_t s);
 void macro_kernel_launch(const MacroArgs& a, cudaStream_t s);
 void tile_kernel_launch(const MacroArgs& a, cudaStream_t s);

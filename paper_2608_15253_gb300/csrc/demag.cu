@@ -940,7 +940,8 @@ static void demag_apply_t(mm_ctx* c, const T* m, T* Hd, int stage = 0, bool c2r 
 // [x], FP32): the 2-D passes of one film run over all of them at once -- the
 // X pass over 3 ny Rc rows, the column convolution over Rc film planes with
 // the shared tensor spectrum (it does not depend on the plane), the inverse
-// X pass -- with the spectrum S laid out [replica][component][PyA][Wk].
+// X pass (Hd == null: left to the caller) -- with the spectrum S laid out
+// [replica][component][PyA][Wk].
 void demag_apply_stacked2d(mm_ctx* c, const DemagPlan& p, const float* m, float* Hd, void* S, int nx, int ny,
                            int Rc) {
     const DemagPlan saved = c->dm;
@@ -966,8 +967,9 @@ void demag_apply_stacked2d(mm_ctx* c, const DemagPlan& p, const float* m, float*
         a.L_other = 1; a.axis_is_y = 1;
         launch_col<float, 0>(c, a, Rc, "fft_conv_stacked", bytes);
     }
-    launch_x<float>(c, false, nullptr, Hd, Sp, 3 * ny * Rc, ny, p.PyA, nx, nx, p.Lh, (const cplx<float>*)p.tw_x,
-                    false, N);
+    if (Hd)
+        launch_x<float>(c, false, nullptr, Hd, Sp, 3 * ny * Rc, ny, p.PyA, nx, nx, p.Lh, (const cplx<float>*)p.tw_x,
+                        false, N);
     c->dm = saved;
 }
 

@@ -182,14 +182,6 @@ bool field_c2r_fusable(const mm_ctx* c) {
     return g.nx % 2 == 0 && g.nx <= c->dm.Lh && field_x_full(c->dm.Lh).group > 0;
 }
 
-// rows per CTA: as many as 96 threads transform at once (at least one; 192
-// threads at 12 warps an SM were slower, see the kernel), fewer on small grids
-// so that two CTAs per SM run
-static int c2r_rows(int G, long long rows, int sms) {
-    const long long want = (rows + 2 * sms - 1) / (2 * sms);
-    return (int)std::max(1LL, std::min<long long>(96 / (3 * G), want));
-}
-
 // opts the kernels of the plan's length into their shared memory and loads
 // them, outside any stream capture
 cudaError_t field_c2r_setup(const mm_ctx* c) {
@@ -219,7 +211,7 @@ void field_c2r_launch(mm_ctx* c, int mode, unsigned terms, const void* m, void* 
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int rpc = c2r_rows(f.group, rows, sms);
+    const int rpc = c2r_rows(f.group, rows);
     const long long grid = (rows + rpc - 1) / rpc;
     const C2RSpec sp{(const float2*)d.spec, (const float2*)d.tw_x, d.PyA, d.Wk, rpc};
     // grids that fill the chip with CTAs of 96 threads: five of them per SM; on

@@ -54,10 +54,20 @@ FieldX field_x_ext(int M);
 
 // threads that transform rpc rows, in whole warps, and the shared memory: their
 // exchange lines, and the field rows over them
-inline int field_x_fft(int group, int rpc) { return (3 * rpc * group + 31) / 32 * 32; }
+constexpr int field_x_fft(int group, int rpc) { return (3 * rpc * group + 31) / 32 * 32; }
 inline size_t field_x_smem(int group, size_t line, int nx, int rpc) {
     const size_t tasks = (field_x_fft(group, rpc) + group - 1) / group;
     return std::max(tasks * line, (size_t)3 * rpc * nx * sizeof(float));
+}
+
+// rows per CTA: as many as 96 threads transform at once (at least one), fewer on
+// small grids so that two CTAs per SM run
+inline int c2r_rows(int G, long long rows) {
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const long long want = (rows + 2 * sms - 1) / (2 * sms);
+    return (int)std::max(1LL, std::min<long long>(96 / (3 * G), want));
 }
 
 template <int M, int G, int Q, int KIND, int V>
@@ -70,7 +80,7 @@ __global__ void __launch_bounds__(kC2RThreads, 3) c2r_field_kernel(FieldArgs<flo
     float* sH = reinterpret_cast<float*>(smem_raw);   // [rpc][3][nx], once the lines are in registers
     const int nx = a.nx, rpc = s.rpc, nrows = a.ny * a.nz;
     const int row0 = blockIdx.x * rpc;
-    if ((int)threadIdx.x < (3 * rpc * G + 31) / 32 * 32) {
+    if ((int)threadIdx.x < field_x_fft(G, rpc)) {
         const int task = threadIdx.x / G, rl = task / 3, comp = task - 3 * rl, row = row0 + rl;
         const bool valid = rl < rpc && row < nrows;
         const int z = valid ? row / a.ny : 0, y = valid ? row - z * a.ny : 0;

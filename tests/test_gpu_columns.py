@@ -201,3 +201,39 @@ def test_small_film_ensembles_match_oracle(n, integrator):
             assert np.abs(mm.mm_get_m(ctx, r, m0[r].shape) - o.m).max() <= 1e-5, (r, n)
     finally:
         mm.mm_destroy(ctx)
+
+
+@pytest.mark.parametrize("integrator", ["heun", "dm"])
+@pytest.mark.parametrize("nx", [12, 16, 20, 24, 28, 32, 36, 44, 52, 60, 64, 72, 80, 96, 108, 128, 140, 160, 192, 212, 240, 256, 260])
+def test_stacked_films_with_the_x_pass_in_the_field_kernel(nx, integrator):
+    """Two size classes in the stacked shape, rows of every length that has the
+    fused kernel (and one above), a temperature and a current per replica, three
+    steps against the FP64 oracle."""
+    mm = need_gpu()
+    from oracle.llg import Solver, Torque
+    mat, cell = W.Material(Ms=1.1e6, A=2e-11, alpha=0.05, Ku1=9e5, D=1e-3), (2e-9, 2e-9, 1e-9)
+    sizes = [(nx, 5)] * 3 + [(9, 7)]
+    M = mm.Material(mat.Ms, mat.A, mat.alpha, mat.Ku1, mat.u, mat.D)
+    cfg = mm.make_config(precision=32, integrator=mm.MM_HEUN if integrator == "heun" else mm.MM_DM,
+                         demag=mm.MM_DEMAG_EXACT, dt=1e-14)
+    seeds = np.arange(1, 5, dtype=np.uint64) * np.uint64(104729)
+    T, J = np.linspace(0.0, 300.0, 4), np.linspace(1e11, 3e11, 4)
+    ctx = mm.mm_create_batch([mm.make_grid(a, b, 1, *cell) for a, b in sizes], M.s, cfg, seeds)
+    try:
+        mm.mm_batch_set_shape(ctx, 0)
+        mm.mm_set_temperature(ctx, T)
+        mm.mm_set_torque(ctx, mm.make_torque(mm.MM_TORQUE_SOT, p=(0, 1, 0), theta_SH=0.1, fl_ratio=0.3), J)
+        g = [W.Grid(a, b, 1, *cell) for a, b in sizes]
+        m0 = [W.m_perp(g[r], seed=nx + r, tilt=0.3) for r in range(4)]
+        for r in range(4):
+            mm.mm_set_m(ctx, r, m0[r])
+        mm.mm_step(ctx, 3)
+        for r in range(4):
+            o = Solver(oracle_problem(g[r], mat), m0[r], terms=("exchange", "dmi", "anisotropy", "zeeman", "demag"), T=T[r],
+                       seed=int(seeds[r]), dt=1e-14,
+                       torque=Torque(kind="sot", J=J[r], p=(0, 1, 0), theta_SH=0.1, fl_ratio=0.3))
+            for _ in range(3):
+                o.heun_step() if integrator == "heun" else o.dm_step()
+            assert np.abs(mm.mm_get_m(ctx, r, m0[r].shape) - o.m).max() <= 1e-5, (r, nx)
+    finally:
+        mm.mm_destroy(ctx)
