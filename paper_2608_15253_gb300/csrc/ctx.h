@@ -208,12 +208,13 @@ struct LaunchScope {
 // demag.cu
 mm_status demag_setup(mm_ctx* c);
 void demag_free(mm_ctx* c);
+int sm_count();   // of the current device
 void demag_apply(mm_ctx* c, const void* m, void* Hd);   // Hd = H_demag(m)
-// FP32 RK45 stage s fused into the X pass: forms m_s = m0 + sum (dt a_sj) k_j
+// RK45 stage s fused into the X pass: forms m_s = m0 + sum (dt a_sj) k_j
 // into d_mtmp while transforming it, then Hd = H_demag(m_s)
 bool demag_stage_fusable(const mm_ctx* c);
 void demag_apply_stage(mm_ctx* c, int stage, void* Hd);
-// FP32: every demag pass but the inverse X pass, for the fused inverse-X +
+// every demag pass but the inverse X pass, for the fused inverse-X +
 // field kernel (stage > 0: the RK45 stage state is formed into d_mtmp first)
 void demag_apply_partial(mm_ctx* c, const void* m, int stage);
 mm_status newell_gpu(long count, const int* ijk, double dx, double dy, double dz, double* out_host);
@@ -228,7 +229,7 @@ void field_launch(mm_ctx* c, int mode, unsigned terms, const void* m, const void
 void thermal_raw_launch(mm_ctx* c, long long step, uint32_t* d_raw, void* d_h);
 // inverse X pass + field kernel in one launch (the demag spectrum of the
 // state must be ready); field_c2r_fusable says whether the grid allows it
-bool field_c2r_fusable(const mm_ctx* c);
+bool field_c2r_fusable(const mm_ctx* c, int mode, unsigned terms);
 cudaError_t field_c2r_setup(const mm_ctx* c);
 void field_c2r_launch(mm_ctx* c, int mode, unsigned terms, const void* m, void* out, void* out2, const void* m0,
                       const void* k1, long long step_override, int gate, int kstage, bool finish = false);

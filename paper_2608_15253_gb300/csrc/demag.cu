@@ -615,7 +615,7 @@ static void* make_twiddles(int L) {
 static int col_threads(int L) { return L >= 512 ? 512 : 256; }
 
 // multiprocessors of the current device (cached per device)
-static int sm_count() {
+int sm_count() {
     static int cache[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
@@ -994,7 +994,9 @@ void demag_apply_stage(mm_ctx* c, int stage, void* Hd) {
 }
 
 void demag_apply_partial(mm_ctx* c, const void* m, int stage) {
-    demag_apply_t<float>(c, (const float*)(stage > 0 ? c->d_mtmp : m), nullptr, stage, false);
+    const void* in = stage > 0 ? c->d_mtmp : m;
+    if (c->prec == 32) demag_apply_t<float>(c, (const float*)in, nullptr, stage, false);
+    else demag_apply_t<double>(c, (const double*)in, nullptr, stage, false);
 }
 
 template <typename T>
@@ -1109,7 +1111,7 @@ static mm_status demag_setup_t(mm_ctx* c) {
     cudaFree(sp);
     free_tw64();
     if (e != cudaSuccess) return cuda_check(c, e, "demag setup");
-    if (sizeof(T) == 4) e = field_c2r_setup(c);
+    e = field_c2r_setup(c);
     if (e != cudaSuccess) return cuda_check(c, e, "field kernel attributes");
     d.on = 1;
     return MM_OK;

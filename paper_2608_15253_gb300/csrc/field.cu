@@ -108,10 +108,8 @@ static FieldArgs<T> field_args(mm_ctx* c, int mode, unsigned terms, const T* m, 
 
 // The QUIET kernels apply: slopes only, no thermal field, no spin torque,
 // none of the further local terms.
-template <typename T>
-static bool field_quiet(const mm_ctx* c, int mode, unsigned terms, const FieldArgs<T>& a) {
-    return mode == MODE_K && !c->ext_terms && a.tq == MM_TORQUE_NONE &&
-           (!(terms & MM_TERM_THERMAL) || a.th_scale == (T)0);
+static bool field_quiet(const mm_ctx* c, int mode, unsigned terms) {
+    return mode == MODE_K && !c->ext_terms && c->tq.kind == MM_TORQUE_NONE && (!(terms & MM_TERM_THERMAL) || !(c->Tr > 0));
 }
 
 static double field_bytes(const mm_ctx* c, int mode, unsigned terms, bool hd) {
@@ -146,7 +144,7 @@ static void field_launch_t(mm_ctx* c, int mode, unsigned terms, const T* m, cons
         if constexpr (sizeof(T) == 4) {
             if (vec) {
                 if (c->ext_terms) launch_dep(field_vec_kernel<kFieldV, true>, grd, blk, 0, c, a);
-                else if (field_quiet(c, mode, terms, a))
+                else if (field_quiet(c, mode, terms))
                     launch_dep(field_vec_kernel<kFieldV, false, true>, grd, blk, 0, c, a);
                 else launch_dep(field_vec_kernel<kFieldV, false>, grd, blk, 0, c, a);
                 return;
@@ -176,18 +174,27 @@ void field_launch(mm_ctx* c, int mode, unsigned terms, const void* m, const void
 // 256x256x16 26.3 us, a 200x50 film 8.7 us (8.1 + 9.4).  Region maps and odd rows
 // take the two kernels: a cell at a time in this one, 150x150x24 with a region
 // map took 44 us against 11.3 + 21.
-bool field_c2r_fusable(const mm_ctx* c) {
+//
+// FP64: slopes alone, and grids of no more rows than SMs (field_fine_d.cu: a row
+// or less per CTA; with more rows the FP64 pipes are busy either way).
+bool field_c2r_fusable(const mm_ctx* c, int mode, unsigned terms) {
     const mm_grid& g = c->grid;
-    if (c->prec != 32 || !c->dm.on || !c->uniform || c->d_region || c->r0f.present == 0.f) return false;
-    return g.nx % 2 == 0 && g.nx <= c->dm.Lh && field_x_full(c->dm.Lh).group > 0;
+    if (!c->dm.on || !c->uniform || c->d_region || g.nx > c->dm.Lh) return false;
+    if (c->prec == 64)
+        return c->r0d.present != 0.0 && field_quiet(c, mode, terms) && (long long)g.ny * g.nz <= sm_count() &&
+               fine_field(c->dm.Lh).kern;
+    return c->r0f.present != 0.f && g.nx % 2 == 0 && field_x_full(c->dm.Lh).group > 0;
 }
 
 // opts the kernels of the plan's length into their shared memory and loads
 // them, outside any stream capture
 cudaError_t field_c2r_setup(const mm_ctx* c) {
     cudaError_t e = cudaSuccess;
-    if (c->prec != 32) return e;
     const int M = c->dm.Lh;
+    if (c->prec == 64) {
+        const FineField f = fine_field(M);
+        return f.kern ? cudaFuncSetAttribute(f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fine_field_smem(f, M, 1)) : e;
+    }
     for (const FieldX& f : {field_x_quiet(M), field_x_full(M), field_x_ext(M)}) {
         if (f.group == 0) continue;
         const size_t smem = field_x_smem(f.group, f.line, M, std::max(1, 96 / (3 * f.group)));
@@ -197,26 +204,40 @@ cudaError_t field_c2r_setup(const mm_ctx* c) {
     return e;
 }
 
+static void fine_field_launch(mm_ctx* c, int mode, unsigned terms, const double* m, double* out, long long step_override,
+                              int gate, int kstage) {
+    const FieldArgs<double> a = field_args<double>(c, mode, terms, m, nullptr, out, nullptr, nullptr, nullptr,
+                                                   step_override, gate, kstage);
+    const DemagPlan& d = c->dm;
+    const int nx = c->grid.nx, rows = c->grid.ny * c->grid.nz;
+    const FineField f = fine_field(d.Lh);
+    const int parts = std::max(1, std::min(sm_count() / rows, (nx + 31) / 32)), warps = std::min(4, ((nx + parts - 1) / parts + 31) / 32);
+    const FineSpec sp{(const double2*)d.spec, (const double2*)d.tw_x, d.PyA, d.Wk, parts};
+    LaunchScope ls(c, "c2r_field", field_bytes(c, mode, terms, false) + 3.0 * rows * (d.Kx * sizeof(double2)));
+    launch_dep(f.kern, rows * parts, 96 + 32 * warps, fine_field_smem(f, nx, parts), c, a, sp);
+}
+
 void field_c2r_launch(mm_ctx* c, int mode, unsigned terms, const void* m, void* out, void* out2, const void* m0,
                       const void* k1, long long step_override, int gate, int kstage, bool finish) {
+    if (c->prec == 64) {
+        fine_field_launch(c, mode, terms, (const double*)m, (double*)out, step_override, gate, kstage);
+        return;
+    }
     FieldArgs<float> a = field_args<float>(c, mode, terms, (const float*)m, nullptr, (float*)out, (float*)out2,
                                            (const float*)m0, (const float*)k1, step_override, gate, kstage);
     if (finish) a.tick = c->d_tick;
     const DemagPlan& d = c->dm;
     const int nx = c->grid.nx;
     const long long rows = (long long)c->grid.ny * c->grid.nz;
-    const bool quiet = !c->ext_terms && field_quiet(c, mode, terms, a);
+    const bool quiet = !c->ext_terms && field_quiet(c, mode, terms);
     const FieldX f = c->ext_terms ? field_x_ext(d.Lh) : quiet ? field_x_quiet(d.Lh) : field_x_full(d.Lh);
     const int four = quiet && nx % 4 == 0;
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int rpc = c2r_rows(f.group, rows);
     const long long grid = (rows + rpc - 1) / rpc;
     const C2RSpec sp{(const float2*)d.spec, (const float2*)d.tw_x, d.PyA, d.Wk, rpc};
     // grids that fill the chip with CTAs of 96 threads: five of them per SM; on
     // smaller ones more threads share the cells (a 512x512 film: 12.0 us against 14.2)
-    const int cells = (rpc * nx / (four ? 4 : 2) + 31) / 32 * 32, most = grid >= 5LL * sms ? 96 : kC2RThreads;
+    const int cells = (rpc * nx / (four ? 4 : 2) + 31) / 32 * 32, most = grid >= 5LL * sm_count() ? 96 : kC2RThreads;
     LaunchScope ls(c, "c2r_field", field_bytes(c, mode, terms, false) + 3.0 * rows * (d.Kx * sizeof(float2)));
     launch_dep(f.kern[four], (unsigned)grid, std::max(field_x_fft(f.group, rpc), std::min(most, cells)),
                field_x_smem(f.group, f.line, nx, rpc), c, a, sp);

@@ -143,6 +143,13 @@ __device__ __forceinline__ void st3(T* a, long long N, long long i, v3<T> v) {
     a[2 * N + i] = v.z;
 }
 
+// LLG torque, Eq. 1: -gamma' mu0 [m x H + alpha m x (m x H)]
+template <typename T>
+__device__ __forceinline__ v3<T> llg_slope(const v3<T>& m, const v3<T>& H, const Region<T>& R) {
+    const v3<T> mxH = cross(m, H);
+    return (-R.gm) * (mxH + R.alpha * cross(m, mxH));
+}
+
 // Effective field of one present cell (x, y, z; linear index i) and, when
 // want_k, its LLG slope with the configured spin torque.  hd is added as the
 // demag field when the caller supplies it (batched path); a.Hd otherwise.
@@ -250,10 +257,8 @@ __device__ __forceinline__ void cell_field_nb(const FieldArgs<T>& a, long long i
         }
     }
     if (!want_k) return;
-    // LLG torque, Eq. 1: -gamma' mu0 [m x H + alpha m x (m x H)]
-    const v3<T> mxH = cross(m, H);
-    if (as_omega) k = R.gm * (H + R.alpha * mxH);
-    else k = (-R.gm) * (mxH + R.alpha * cross(m, mxH));
+    if (as_omega) k = R.gm * (H + R.alpha * cross(m, H));
+    else k = llg_slope(m, H, R);
     if (QUIET) return;
     if (a.tq == MM_TORQUE_SOT || a.tq == MM_TORQUE_STT) {
         const v3<T> p = mk3<T>(a.p[0], a.p[1], a.p[2]);
@@ -353,13 +358,13 @@ __device__ __forceinline__ v3<T> ghost_value(const v3<T>& m, int d, int sg, T h,
 // rotation vector, see cell_field_nb).  UNIF: one material
 // everywhere (no region map): every in-grid neighbour is present and every
 // exchange pair uses the one coefficient a.c_uniform.
-template <typename T, bool UNIF = false, bool EXT = true>
+template <typename T, bool UNIF = false, bool EXT = true, bool QUIET = false>
 __device__ __forceinline__ void cell_field(const FieldArgs<T>& a, int x, int y, int z, long long i, int ri,
                                            const Region<T>& R, const v3<T>& m, const v3<T>* hd, long long step,
                                            v3<T>& H, v3<T>& k, bool want_k, bool as_omega = false) {
     const long long N = a.N;
     const unsigned nbt = MM_TERM_EXCHANGE | MM_TERM_DMI | (EXT ? MM_TERM_SURFACE : 0u);
-    const bool need_nb = (a.terms & nbt) || a.tq == MM_TORQUE_ZL;
+    const bool need_nb = (a.terms & nbt) || (!QUIET && a.tq == MM_TORQUE_ZL);
     // neighbour values (ghosts where absent) and raw presence (Zhang-Li,
     // the free faces of the surface term)
     v3<T> nbv[6];
@@ -403,8 +408,8 @@ __device__ __forceinline__ void cell_field(const FieldArgs<T>& a, int x, int y, 
             }
         }
     }
-    cell_field_nb<T, EXT>(a, i, R, m, nbv, nbp, cnb, hd != nullptr, hd ? *hd : mk3<T>(0, 0, 0), step, H, k, want_k,
-                     as_omega);
+    cell_field_nb<T, EXT, QUIET>(a, i, R, m, nbv, nbp, cnb, hd != nullptr, hd ? *hd : mk3<T>(0, 0, 0), step, H, k,
+                                 want_k, as_omega);
 }
 
 }  // namespace mm

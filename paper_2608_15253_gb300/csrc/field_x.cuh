@@ -63,11 +63,25 @@ inline size_t field_x_smem(int group, size_t line, int nx, int rpc) {
 // rows per CTA: as many as 96 threads transform at once (at least one), fewer on
 // small grids so that two CTAs per SM run
 inline int c2r_rows(int G, long long rows) {
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long want = (rows + 2 * sms - 1) / (2 * sms);
+    const long long want = (rows + 2 * sm_count() - 1) / (2 * sm_count());
     return (int)std::max(1LL, std::min<long long>(96 / (3 * G), want));
+}
+
+// The same for small FP64 grids (field_fine_d.cu).
+struct FineSpec {
+    const double2* spec;    // [3][nz][PyA][Wk]
+    const double2* tw;      // exp(-2 pi i q / Px)
+    int PyA, Wk;
+    int parts;              // CTAs per row
+};
+struct FineField {
+    void (*kern)(FieldArgs<double>, FineSpec) = nullptr;
+    size_t line = 0;        // bytes of a component's line
+};
+FineField fine_field(int M);
+constexpr int kFineFieldThreads = 224;   // three warps of transforms, up to four of cells
+inline size_t fine_field_smem(const FineField& f, int nx, int parts) {
+    return 3 * f.line + 3 * sizeof(double) * (nx + (nx + parts - 1) / parts);
 }
 
 template <int M, int G, int Q, int KIND, int V>

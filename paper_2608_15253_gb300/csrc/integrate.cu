@@ -251,7 +251,7 @@ void demag_eval(mm_ctx* c, const void* m, void* Hd) {
 // field kernel and H_demag never goes through global memory.
 static void demag_and_field(mm_ctx* c, bool demag, int mode, unsigned terms, const void* m, void* out, void* out2,
                             const void* m0, const void* k1, int gate, int kstage, bool finish = false) {
-    if (demag && !surrogate_active(c) && field_c2r_fusable(c)) {
+    if (demag && !surrogate_active(c) && field_c2r_fusable(c, mode, terms)) {
         demag_apply_partial(c, m, 0);
         field_c2r_launch(c, mode, terms, m, out, out2, m0, k1, -1, gate, kstage, finish);
         return;
@@ -272,7 +272,7 @@ static void rk45_attempt_t(mm_ctx* c) {
     const unsigned terms = c->terms;
     const bool demag = c->dm.on && (terms & MM_TERM_DEMAG);
     const bool fused = demag && !surrogate_active(c) && demag_stage_fusable(c);
-    const bool fused_c2r = fused && field_c2r_fusable(c);
+    const bool fused_c2r = fused && field_c2r_fusable(c, MODE_K, terms);
     for (int s = 1; s < 7; ++s) {
         if (fused_c2r) {
             // stage combine inside the forward X pass, inverse X pass inside the field kernel

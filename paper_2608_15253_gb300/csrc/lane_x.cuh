@@ -450,6 +450,22 @@ __global__ void __launch_bounds__(128) fine_r2c_kernel(XLaneArgs<T> a) {
     }
 }
 
+// Half spectrum of one row to store(n, (x[2n], x[2n+1])), by one warp; sm: the
+// row's fine_line values.
+template <typename T, int M, typename Store>
+__device__ __forceinline__ void fine_c2r_row(const cplx<T>* X, const cplx<T>* __restrict__ tw, lcx<T>* sm, Store store) {
+    for (int k = threadIdx.x & 31; k <= M / 2; k += 32) {
+        lcx<T> z, zm;
+        x_merge<T>(X[k], X[M - k], __ldg(tw + k), z, zm);
+        sm[fine_at(k)] = z;
+        if (k > 0 && 2 * k != M) sm[fine_at(M - k)] = zm;
+    }
+    __syncwarp();
+    constexpr int NP = fine_npass(M);
+    fine_passes<T, -1, M, 0, NP - 1>(sm, tw);
+    fine_pass<T, -1, M, NP - 1>(tw, [&](int i) { return sm[fine_at(i)]; }, store);
+}
+
 template <typename T, int M>
 __global__ void __launch_bounds__(128) fine_c2r_kernel(XLaneArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -458,17 +474,8 @@ __global__ void __launch_bounds__(128) fine_c2r_kernel(XLaneArgs<T> a) {
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= a.rows) return;                                    // whole warp
     const cplx<T>* X = a.spec + ((long long)(row / a.rows_per_plane) * a.spec_rows_per_plane + row % a.rows_per_plane) * a.Wk;
-    for (int k = threadIdx.x & 31; k <= M / 2; k += 32) {
-        lcx<T> z, zm;
-        x_merge<T>(X[k], X[M - k], __ldg(a.tw + k), z, zm);
-        sm[fine_at(k)] = z;
-        if (k > 0 && 2 * k != M) sm[fine_at(M - k)] = zm;
-    }
-    __syncwarp();
-    constexpr int NP = fine_npass(M);
-    fine_passes<T, -1, M, 0, NP - 1>(sm, a.tw);
     T* out = a.out + (long long)row * a.nx;
-    fine_pass<T, -1, M, NP - 1>(a.tw, [&](int i) { return sm[fine_at(i)]; }, [&](int n, lcx<T> v) {
+    fine_c2r_row<T, M>(X, a.tw, sm, [&](int n, lcx<T> v) {
         if (2 * n < a.nx) out[2 * n] = v.re;
         if (2 * n + 1 < a.nx) out[2 * n + 1] = v.im;
     });

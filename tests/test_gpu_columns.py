@@ -165,6 +165,28 @@ def test_x_pass_inside_the_field_kernel(L, kind):
             mm.mm_destroy(ctx)
 
 
+@pytest.mark.parametrize("L", X_LENGTHS)
+def test_x_pass_inside_the_fp64_slopes(L):
+    """FP64 rows padded to L, even and odd, few enough that CTAs share a row: two
+    RK4 steps and two RK45 steps of the oracle's sizes."""
+    mm = need_gpu()
+    from oracle.llg import Solver
+    below = max([v for v in LENGTHS if v % 2 == 0 and v < L])
+    for nx in sorted({below // 2 + 1, L // 2 - 1, L // 2} - {1}):
+        grid = W.Grid(nx, 5, 2, 2e-9, 2e-9, 2e-9)
+        m0 = W.m_perp(grid, seed=nx, tilt=0.3)
+        for integrator in ("rk4", "rk45"):
+            o = Solver(oracle_problem(grid, MAT), m0, terms=("exchange", "zeeman", "demag"), dt=1e-14, rtol=1e-6)
+            dts = [(o.rk4_step(), 1e-14)[1] if integrator == "rk4" else o.rk45_step() for _ in range(2)]
+            ctx = make_ctx(mm, grid, MAT, precision=64, dt=1e-14, rtol=1e-6, integrator=integrator)
+            try:
+                mm.mm_set_m(ctx, 0, m0)
+                mm.mm_step(ctx, 2) if integrator == "rk4" else mm.mm_step_dt(ctx, dts)
+                assert np.abs(mm.mm_get_m(ctx, 0, m0.shape) - o.m).max() <= 1e-11, (nx, integrator)
+            finally:
+                mm.mm_destroy(ctx)
+
+
 @pytest.mark.parametrize("integrator", ["heun", "dm"])
 @pytest.mark.parametrize("n", [(8, 8), (7, 8), (12, 12), (16, 16), (15, 16), (16, 15), (24, 24), (32, 32), (31, 32)])
 def test_small_film_ensembles_match_oracle(n, integrator):
