@@ -6,7 +6,7 @@
 //   X[k1 + Q k2] = sum_t W_G^(t k2) [ W_L^(t k1) sum_q x[q G + t] W_Q^(q k1) ]
 //
 // Columns are flattened (other-axis index, kx) positions, TP lanes of them
-// (two columns each in FP32) per CTA.  Kernels: the middle pass of 3-D grids
+// (one column each, or two packed ones in FP32) per CTA.  Kernels: the middle pass of 3-D grids
 // and of ensembles of films (lane_conv_kernel), the middle pass of single
 // films (lane_film_kernel), and the Y passes of 3-D grids
 // (lane_col_kernel).  Each kernel's comment gives its split.

@@ -1,15 +1,18 @@
 // Open-boundary demagnetisation (Methods, "Physics and discretization":
 // FFT convolution with the Newell tensor, zero-padded to 2N).
 //
-// Pipeline per field evaluation, every pass a shared-memory batched FFT:
+// Pipeline per field evaluation; a pass is a register FFT over lanes with one
+// shared-memory exchange (fft_lane.cuh) where its length has a kernel, a
+// runtime-planned shared-memory FFT (fft_rt.cuh) elsewhere:
 //   X pass   R2C along x of Ms*m (only the nx nonzero inputs of the padded
 //            2nx row are read; half-length complex FFT + split)
 //   Y pass   forward along y (3-D only; ny nonzero inputs, Py outputs)
 //   middle   last axis (z in 3-D, y in 2-D): forward FFT, H^ = K^ M^ with the
 //            real, symmetry-compressed tensor spectrum, inverse FFT, keep the
-//            n un-padded outputs -- one pass, the spectrum never leaves smem
+//            n un-padded outputs -- one pass
 //   Y pass   inverse (3-D only; Py inputs, ny outputs)
-//   X pass   C2R, only the nx un-padded outputs are written.
+//   X pass   C2R, only the nx un-padded outputs are written (inside the field
+//            kernel where field_x.cuh has a form for the grid).
 // Setup (once per geometry): the FP64 Newell tensor on the GPU (closed form
 // near, tent-weighted Gauss-Legendre of the dipole kernel far), then FP64
 // FFTs of the padded tensor; -1/(Px Py Pz) is folded into K^.
