@@ -990,12 +990,21 @@ static mm_status advance(mm_ctx* c, long long add_steps, double t_end, int repla
     // fixed-step schemes: every attempt is accepted
     const bool heun = c->integrator != MM_RK45 && c->integrator != MM_DM_ADAPTIVE;
     if (c->batch && batch_is_fused(c->batch)) {
-        // one-cell replicas: blocks of fused steps, no graph needed
+        // one-cell replicas and small films: blocks of fused steps, no graph needed
+        const bool sums = add_steps < 0 && batch_sums_time(c->batch);
+        const double dt = c->h_state.dt;
+        double t = c->h_state.t;
         long long want = add_steps >= 0 ? add_steps
-                                        : (long long)std::ceil((t_end - c->h_state.t) / c->h_state.dt);
+                         : sums         ? std::numeric_limits<long long>::max()
+                                        : (long long)std::ceil((t_end - t) / dt);
         while (want > 0) {
-            const int k = (int)std::min<long long>(want, kMacroBlock);
-            batch_macro_steps(c, c->batch, k);
+            int k = (int)std::min<long long>(want, kMacroBlock);
+            if (sums) {   // one more step while t < t_end, t as the steps sum it
+                k = 0;
+                for (double u = t; k < kMacroBlock && u < t_end && u + dt > u; ++k) u += dt;
+                if (k == 0) break;
+            }
+            batch_macro_steps(c, c->batch, k, &t);
             want -= k;
         }
         s = cuda_check(c, cudaGetLastError(), "launch");

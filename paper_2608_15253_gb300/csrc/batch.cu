@@ -298,9 +298,17 @@ static void launch_stage(mm_ctx* c, BatchHost* b, int stage) {
 // picks for them; the persistent shape stays what the caller asked for.
 bool batch_is_fused(BatchHost* b) { return b->macro || b->tile || (b->tile_demag && b->stacked); }
 
+// Ensembles with demag count their time step by step in every launch shape, t
+// rounded after each; those without demag advance by whole blocks, n dt at a time.
+bool batch_sums_time(BatchHost* b) { return b->tile_demag; }
+
 // one launch of `nsteps` fused steps of every replica (one-cell or small
-// films without demag), then the step bookkeeping
-void batch_macro_steps(mm_ctx* c, BatchHost* b, int nsteps) {
+// films), then the step bookkeeping; *t: the time before and after them, where
+// it is summed step by step
+void batch_macro_steps(mm_ctx* c, BatchHost* b, int nsteps, double* t) {
+    const bool sums = batch_sums_time(b);
+    if (sums)
+        for (int s = 0; s < nsteps; ++s) *t += c->h_state.dt;
     MacroArgs a{};
     a.rep = b->d_rep;
     a.R = (int)b->rep.size();
@@ -325,7 +333,7 @@ void batch_macro_steps(mm_ctx* c, BatchHost* b, int nsteps) {
         else tile_demag_launch(a, b->d_cls, b->cls[0].Lh, b->cls[0].Py, c->stream);
     }
     LaunchScope ls(c, "macro_advance", 0.0);
-    macro_advance_launch(c->d_state, nsteps, c->stream);
+    macro_advance_launch(c->d_state, nsteps, sums ? t : nullptr, c->stream);
 }
 
 // Retire/refill (Results, "Replica batching"): trial tables, results, and

@@ -473,7 +473,7 @@ cudaError_t tile_kernel_attributes();
 bool tile_demag_supported(int Lh, int Py);
 cudaError_t tile_demag_attributes(int Lh, int Py);
 void tile_demag_launch(const MacroArgs& a, const ClsDev* cls, int Lh, int Py, cudaStream_t s);
-void macro_advance_launch(DevState* st, int nsteps, cudaStream_t s);
+void macro_advance_launch(DevState* st, int nsteps, const double* t, cudaStream_t s);
 
 // host wrappers, one set per instantiated thread count
 cudaError_t batch_kernel_attributes_256();

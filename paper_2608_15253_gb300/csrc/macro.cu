@@ -382,9 +382,10 @@ void tile_kernel_launch(const MacroArgs& a, cudaStream_t s) {
     else tile_kernel<false><<<a.R, nt, 6 * a.nmax * sizeof(float), s>>>(a);
 }
 
-// fixed-step bookkeeping of a block of n steps
-__global__ void macro_advance_kernel(DevState* st, int n) {
-    st->t += n * st->dt;
+// fixed-step bookkeeping of a block of n steps, to the time t where it is given
+__global__ void macro_advance_kernel(DevState* st, int n, bool given, double t) {
+    if (given) st->t = t;
+    else st->t += n * st->dt;
     st->step += n;
     st->accepted += n;
     st->attempts += n;
@@ -397,8 +398,8 @@ void macro_kernel_launch(const MacroArgs& a, cudaStream_t s) {
     else macro_lean_kernel<<<(a.R + nt - 1) / nt, nt * (1 + kDrawWarps), 0, s>>>(a);
 }
 
-void macro_advance_launch(DevState* st, int nsteps, cudaStream_t s) {
-    macro_advance_kernel<<<1, 1, 0, s>>>(st, nsteps);
+void macro_advance_launch(DevState* st, int nsteps, const double* t, cudaStream_t s) {
+    macro_advance_kernel<<<1, 1, 0, s>>>(st, nsteps, t != nullptr, t ? *t : 0.0);
 }
 
 }  // namespace mm

@@ -1,0 +1,45 @@
+"""Ensembles of one small film size with demag in the stacked shape, which run
+blocks of steps per launch (batch_tile.cu): what a caller sees of the clock and
+of the launch shape is that of every other ensemble with demag."""
+import numpy as np
+import pytest
+
+import workloads as W
+from gpu_util import need_gpu
+
+pytestmark = pytest.mark.gpu
+
+CELL = (2e-9, 2e-9, 1e-9)
+MAT = W.Material(Ms=1.1e6, A=2e-11, alpha=0.05, Ku1=9e5)
+
+
+def _films(mm, n, R, dt, shape=0, integrator=None, T=0.0):
+    M = mm.Material(MAT.Ms, MAT.A, MAT.alpha, MAT.Ku1, MAT.u)
+    cfg = mm.make_config(precision=32, integrator=mm.MM_HEUN if integrator is None else integrator,
+                         demag=mm.MM_DEMAG_EXACT, dt=dt, T=T)
+    ctx = mm.mm_create_batch([mm.make_grid(n, n, 1, *CELL)] * R, M.s, cfg)
+    ctx._mat = M
+    mm.mm_batch_set_shape(ctx, shape, R if shape else 0)
+    return ctx
+
+
+@pytest.mark.parametrize("dt, t_end", [(1e-14, 1e-13), (1e-13, 1e-12), (1e-14, 2e-11)])
+@pytest.mark.parametrize("shape", [0, 256])
+def test_a_run_to_a_time_steps_while_the_summed_time_is_below_it(shape, dt, t_end):
+    """t grows by dt a step, rounded each time, and a step is taken while it is
+    below t_end: 11, 10 and 2001 steps here (ten times 1e-14 is below 1e-13)."""
+    mm = need_gpu()
+    t, n = 0.0, 0
+    while t < t_end:
+        t, n = t + dt, n + 1
+    ctx = _films(mm, 16, 3, dt, shape)
+    try:
+        mm.mm_run(ctx, t_end)
+        assert mm.mm_get_time(ctx) == (t, dt, n)
+        mm.mm_run(ctx, t_end)                       # there already
+        mm.mm_step(ctx, 5)
+        for _ in range(5):
+            t += dt
+        assert mm.mm_get_time(ctx) == (t, dt, n + 5)
+    finally:
+        mm.mm_destroy(ctx)
