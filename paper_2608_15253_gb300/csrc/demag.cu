@@ -76,7 +76,7 @@ __device__ __forceinline__ T stage_value(const XArgs<T>& a, int S, int kf, long 
     for (int j = 0; j < S; ++j) {
         if (j == 1 && S == 6) continue;             // a_7,2 = 0
         const int slot = j == 0 ? kf : j == 6 ? 6 - kf : j;
-        acc += cf[j] * __ldg(a.kptr[slot] + q);
+        acc += cf[j] * a.kptr[slot][q];
     }
     return acc;
 }

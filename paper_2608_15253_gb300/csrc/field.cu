@@ -35,7 +35,11 @@ __global__ void __launch_bounds__(256) field_vec_kernel(FieldArgs<float> a) {
     if (a.gate && !a.st->active) return;
     const int x0 = V * (blockIdx.x * blockDim.x + threadIdx.x);
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x0 < a.nx && y < a.ny) field_vec_cells<V, EXT, false, QUIET>(a, x0, y, blockIdx.z, nullptr, 0);
+    if (x0 < a.nx && y < a.ny) {
+        VecIn<V> in;
+        field_vec_load<V, EXT, QUIET>(a, x0, y, blockIdx.z, in);
+        field_vec_finish<V, EXT, false, QUIET>(a, x0, y, blockIdx.z, in, nullptr, 0);
+    }
     if (!QUIET && a.tick) fixed_finish(const_cast<DevState*>(a.st), a.tick);
 }
 

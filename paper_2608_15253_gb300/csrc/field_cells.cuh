@@ -89,7 +89,7 @@ template <> struct fvec<4> { using t = float4; };
 
 template <int V>
 __device__ __forceinline__ typename fvec<V>::t ldv(const float* p) {
-    return __ldg(reinterpret_cast<const typename fvec<V>::t*>(p));
+    return *reinterpret_cast<const typename fvec<V>::t*>(p);
 }
 template <int V>
 __device__ __forceinline__ void stv(float* p, const typename fvec<V>::t& v) {
@@ -102,30 +102,29 @@ __device__ __forceinline__ void fset(float4& v, int q, float x) {
     if (q == 0) v.x = x; else if (q == 1) v.y = x; else if (q == 2) v.z = x; else v.w = x;
 }
 
-// The V cells x0 .. x0 + V - 1 of row (z, y).  HD_SMEM: the demag field of
-// the cells comes from shared memory (hds[c * hd_stride + q], the fused
-// inverse-X-pass kernel below), else from a.Hd in global memory.  QUIET:
-// slopes only (MODE_K), no thermal field, no spin torque -- the variant for
-// deterministic runs without current, with far fewer registers.
-template <int V, bool EXT, bool HD_SMEM, bool QUIET = false>
-__device__ __forceinline__ void field_vec_cells(const FieldArgs<float>& a, int x0, int y, int z, const float* hds,
-                                                int hd_stride) {
+// What V cells x0 .. x0 + V - 1 of row (z, y) need of the state: themselves and
+// their neighbours.  Read on its own, so that the fused kernel's idle threads can
+// do it ahead of the barrier that brings the demag field: plain loads are not
+// moved across it.
+template <int V>
+struct VecIn {
     using VT = typename fvec<V>::t;
+    VT m[3], nr[4][3];              // the cells; the neighbour rows y+, y-, z+, z-
+    float xl[3], xr[3];             // the two row-end x neighbours
+    bool rin[4], lin, rinx;
+};
+
+template <int V, bool EXT, bool QUIET>
+__device__ __forceinline__ void field_vec_load(const FieldArgs<float>& a, int x0, int y, int z, VecIn<V>& in) {
     const long long N = a.N;
     const long long i0 = ((long long)z * a.ny + y) * a.nx + x0;
-    const Region<float>& R = a.R0;
-    const long long step = a.step_override >= 0 ? a.step_override : (a.st ? a.st->step : 0);
-    VT mc[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) mc[c] = ldv<V>(a.m + c * N + i0);
+    for (int c = 0; c < 3; ++c) in.m[c] = ldv<V>(a.m + c * N + i0);
     const unsigned nbt = MM_TERM_EXCHANGE | MM_TERM_DMI | (EXT ? MM_TERM_SURFACE : 0u);
-    const bool need_nb = (a.terms & nbt) || (!QUIET && a.tq == MM_TORQUE_ZL);
-    // neighbour rows (y+, y-, z+, z-) as vectors, row-end x neighbours as scalars
-    VT nr[4][3];
-    bool rin[4] = {false, false, false, false};
-    float xl[3] = {0, 0, 0}, xr[3] = {0, 0, 0};
-    bool lin = false, rinx = false;
-    if (need_nb) {
+    in.lin = in.rinx = false;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) in.rin[s] = false;
+    if ((a.terms & nbt) || (!QUIET && a.tq == MM_TORQUE_ZL)) {
         const long long sy = a.nx, sz = (long long)a.nx * a.ny;
         const int ny = a.ny, nz = a.nz;
         const int qs[4] = {y + 1, y - 1, z + 1, z - 1};
@@ -138,23 +137,61 @@ __device__ __forceinline__ void field_vec_cells(const FieldArgs<float>& a, int x
             int q = qs[s];
             bool inside = q >= 0 && q < dm[s];
             if (!inside && pr[s]) { q = (q + dm[s]) % dm[s]; inside = true; }
-            rin[s] = inside;
+            in.rin[s] = inside;
             if (inside) {
                 const long long j = i0 + (long long)(q - ps[s]) * st[s];
 #pragma unroll
-                for (int c = 0; c < 3; ++c) nr[s][c] = ldv<V>(a.m + c * N + j);
+                for (int c = 0; c < 3; ++c) in.nr[s][c] = ldv<V>(a.m + c * N + j);
             }
         }
         int ql = x0 - 1, qr = x0 + V;
-        lin = ql >= 0;
-        rinx = qr < a.nx;
-        if (!lin && a.px) { ql += a.nx; lin = true; }
-        if (!rinx && a.px) { qr -= a.nx; rinx = true; }
+        in.lin = ql >= 0;
+        in.rinx = qr < a.nx;
+        if (!in.lin && a.px) { ql += a.nx; in.lin = true; }
+        if (!in.rinx && a.px) { qr -= a.nx; in.rinx = true; }
         const long long row = i0 - x0;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            if (lin) xl[c] = __ldg(a.m + c * N + row + ql);
-            if (rinx) xr[c] = __ldg(a.m + c * N + row + qr);
+            if (in.lin) in.xl[c] = a.m[c * N + row + ql];
+            if (in.rinx) in.xr[c] = a.m[c * N + row + qr];
+        }
+    }
+}
+
+// The output of these cells.  HD_SMEM: their demag field comes from shared
+// memory (hds[c * hd_stride + q], the fused inverse-X-pass kernel), else from
+// a.Hd in global memory.  QUIET: slopes only (MODE_K), no thermal field, no spin
+// torque -- the variant for deterministic runs without current, with far fewer
+// registers.  What a mode reads and writes beside the slope is done for all cells
+// together: a cell at a time, a corrector's loads wait for the store of the other
+// cell's thermal field, and a small grid for its instructions.  512x512x32 Heun
+// without demag 291 -> 272 us a step, at 300 K 386 -> 336; with demag 1755 -> 1692;
+// 256x256 films 36.3 -> 36.7 (the price of plain loads there, 37.8 without this).
+template <int V, bool EXT, bool HD_SMEM, bool QUIET>
+__device__ __forceinline__ void field_vec_finish(const FieldArgs<float>& a, int x0, int y, int z, const VecIn<V>& in,
+                                                 const float* hds, int hd_stride) {
+    using VT = typename fvec<V>::t;
+    const long long N = a.N;
+    const long long i0 = ((long long)z * a.ny + y) * a.nx + x0;
+    const Region<float>& R = a.R0;
+    const unsigned nbt = MM_TERM_EXCHANGE | MM_TERM_DMI | (EXT ? MM_TERM_SURFACE : 0u);
+    const bool need_nb = (a.terms & nbt) || (!QUIET && a.tq == MM_TORQUE_ZL);
+    VT th[3];
+    if (!QUIET && (a.terms & MM_TERM_THERMAL) && a.th_scale != 0.f) {
+        if (a.noise && (a.mode == MODE_HEUN2 || a.mode == MODE_DM2)) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) th[c] = ldv<V>(a.noise + c * N + i0);
+        } else {
+            const long long step = a.step_override >= 0 ? a.step_override : (a.st ? a.st->step : 0);
+#pragma unroll
+            for (int q = 0; q < V; ++q) {
+                const v3<float> t = thermal_h<float>(a, i0 + q, a.R0, step);
+                fset(th[0], q, t.x); fset(th[1], q, t.y); fset(th[2], q, t.z);
+            }
+            if (a.noise) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) stv<V>(a.noise + c * N + i0, th[c]);
+            }
         }
     }
     VT hd[3];
@@ -164,63 +201,69 @@ __device__ __forceinline__ void field_vec_cells(const FieldArgs<float>& a, int x
         for (int c = 0; c < 3; ++c)
             hd[c] = HD_SMEM ? *reinterpret_cast<const VT*>(hds + c * hd_stride) : ldv<V>(a.Hd + c * N + i0);
     }
+    auto get = [](const VT* v, int q) { return mk3<float>(fget(v[0], q), fget(v[1], q), fget(v[2], q)); };
     VT o1[3], o2[3];
+    auto put = [&](int q, const v3<float>& r) { fset(o1[0], q, r.x); fset(o1[1], q, r.y); fset(o1[2], q, r.z); };
 #pragma unroll
     for (int q = 0; q < V; ++q) {
-        const v3<float> m = mk3<float>(fget(mc[0], q), fget(mc[1], q), fget(mc[2], q));
+        const v3<float> m = get(in.m, q);
         v3<float> nbv[6];
         bool nbp[6];
         float cnb[6];
         if (need_nb) {
             // x+ / x-
-            const bool pp = q < V - 1 || rinx, pm = q > 0 || lin;
+            const bool pp = q < V - 1 || in.rinx, pm = q > 0 || in.lin;
             nbp[0] = pp;
             nbp[1] = pm;
-            nbv[0] = q < V - 1 ? mk3<float>(fget(mc[0], q + 1), fget(mc[1], q + 1), fget(mc[2], q + 1))
-                               : (rinx ? mk3<float>(xr[0], xr[1], xr[2]) : ghost_value<float, EXT>(m, 0, 1, a.hx, R.ratio, R.ratio_b));
-            nbv[1] = q > 0 ? mk3<float>(fget(mc[0], q - 1), fget(mc[1], q - 1), fget(mc[2], q - 1))
-                           : (lin ? mk3<float>(xl[0], xl[1], xl[2]) : ghost_value<float, EXT>(m, 0, -1, a.hx, R.ratio, R.ratio_b));
+            nbv[0] = q < V - 1 ? get(in.m, q < V - 1 ? q + 1 : q)
+                               : (in.rinx ? mk3<float>(in.xr[0], in.xr[1], in.xr[2]) : ghost_value<float, EXT>(m, 0, 1, a.hx, R.ratio, R.ratio_b));
+            nbv[1] = q > 0 ? get(in.m, q > 0 ? q - 1 : q)
+                           : (in.lin ? mk3<float>(in.xl[0], in.xl[1], in.xl[2]) : ghost_value<float, EXT>(m, 0, -1, a.hx, R.ratio, R.ratio_b));
             cnb[0] = pp ? a.c_uniform : R.cg;
             cnb[1] = pm ? a.c_uniform : R.cg;
 #pragma unroll
             for (int s = 0; s < 4; ++s) {
                 const int slot = 2 + s, d = 1 + s / 2, sg = (s & 1) ? -1 : 1;
-                nbp[slot] = rin[s];
-                nbv[slot] = rin[s] ? mk3<float>(fget(nr[s][0], q), fget(nr[s][1], q), fget(nr[s][2], q))
-                                   : ghost_value<float, EXT>(m, d, sg, d == 1 ? a.hy : a.hz, R.ratio, R.ratio_b);
-                cnb[slot] = rin[s] ? a.c_uniform : R.cg;
+                nbp[slot] = in.rin[s];
+                nbv[slot] = in.rin[s] ? get(in.nr[s], q)
+                                      : ghost_value<float, EXT>(m, d, sg, d == 1 ? a.hy : a.hz, R.ratio, R.ratio_b);
+                cnb[slot] = in.rin[s] ? a.c_uniform : R.cg;
             }
         }
-        const v3<float> hq = dem ? mk3<float>(fget(hd[0], q), fget(hd[1], q), fget(hd[2], q)) : mk3<float>(0, 0, 0);
+        const v3<float> hq = dem ? get(hd, q) : mk3<float>(0, 0, 0), thq = get(th, q);
         v3<float> H, k;
-        cell_field_nb<float, EXT, QUIET>(a, i0 + q, R, m, nbv, nbp, cnb, dem, hq, step, H, k,
-                                         QUIET || a.mode != MODE_H, !QUIET && a.mode >= MODE_DM1);
-        v3<float> r1 = H, r2 = k;
-        if (QUIET || a.mode == MODE_K) r1 = k;
-        else if (QUIET) {
-        } else if (a.mode == MODE_HEUN1) {
-            const float dt = (float)a.st->dt_eff;
-            r1 = m + dt * k;
-            r2 = k;
-        } else if (a.mode == MODE_HEUN2) {
-            const float dt = (float)a.st->dt_eff;
-            const long long i = i0 + q;
-            const v3<float> m0 = ld3(a.m0, N, i);
-            const v3<float> k1 = ld3(a.k1, N, i);
-            v3<float> mn = m0 + (0.5f * dt) * (k1 + k);
-            r1 = (1.0f / sqrtf(dot(mn, mn))) * mn;
+        cell_field_nb<float, EXT, QUIET>(a, i0 + q, R, m, nbv, nbp, cnb, dem, hq, 0, H, k, QUIET || HD_SMEM || a.mode != MODE_H,
+                                         !QUIET && a.mode >= MODE_DM1, &thq);
+        put(q, QUIET ? k : H);
+        if (!QUIET) { fset(o2[0], q, k.x); fset(o2[1], q, k.y); fset(o2[2], q, k.z); }
+    }
+    // the stage's output of all cells, the mode looked up once
+    if (QUIET) {
+    } else if (a.mode == MODE_K) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) o1[c] = o2[c];
+    } else if (HD_SMEM || a.mode != MODE_H) {
+        const float dt = (float)a.st->dt_eff;
+        if (a.mode == MODE_HEUN1) {
+#pragma unroll
+            for (int q = 0; q < V; ++q) put(q, get(in.m, q) + dt * get(o2, q));
         } else if (a.mode == MODE_DM1) {
-            r1 = rodrigues<float>(m, k, (float)a.st->dt_eff);
-            r2 = k;
-        } else if (a.mode == MODE_DM2) {
-            const long long i = i0 + q;
-            const v3<float> m0 = ld3(a.m0, N, i);
-            const v3<float> w1 = ld3(a.k1, N, i);
-            const v3<float> mn = rodrigues<float>(m0, 0.5f * (w1 + k), (float)a.st->dt_eff);
-            r1 = (1.0f / sqrtf(dot(mn, mn))) * mn;
+#pragma unroll
+            for (int q = 0; q < V; ++q) put(q, rodrigues<float>(get(in.m, q), get(o2, q), dt));
+        } else {
+            VT b0[3], b1[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                b0[c] = ldv<V>(a.m0 + c * N + i0);
+                b1[c] = ldv<V>(a.k1 + c * N + i0);
+            }
+#pragma unroll
+            for (int q = 0; q < V; ++q) {
+                const v3<float> m0 = get(b0, q), kk = get(b1, q) + get(o2, q);
+                const v3<float> mn = a.mode == MODE_HEUN2 ? m0 + (0.5f * dt) * kk : rodrigues<float>(m0, 0.5f * kk, dt);
+                put(q, (1.0f / sqrtf(dot(mn, mn))) * mn);
+            }
         }
-        fset(o1[0], q, r1.x); fset(o1[1], q, r1.y); fset(o1[2], q, r1.z);
-        fset(o2[0], q, r2.x); fset(o2[1], q, r2.y); fset(o2[2], q, r2.z);
     }
     float* o = a.out;
     if (!o) {

@@ -132,8 +132,8 @@ __device__ __forceinline__ v3<T> thermal_h(const FieldArgs<T>& a, long long i, c
 }
 
 template <typename T>
-__device__ __forceinline__ v3<T> ld3(const T* __restrict__ a, long long N, long long i) {
-    return mk3<T>(__ldg(a + i), __ldg(a + N + i), __ldg(a + 2 * N + i));
+__device__ __forceinline__ v3<T> ld3(const T* a, long long N, long long i) {
+    return mk3<T>(a[i], a[N + i], a[2 * N + i]);
 }
 
 template <typename T>
@@ -169,12 +169,13 @@ __device__ __forceinline__ v3<T> llg_slope(const v3<T>& m, const v3<T>& H, const
 // EXT = false compiles out bulk DMI and the further local terms (cubic,
 // surface, RKKY, magnetoelastic): the lean kernel for contexts without them.
 // QUIET = true also compiles out the thermal field and every spin torque
-// (contexts at T = 0 without current).
+// (contexts at T = 0 without current).  th: the thermal field, where the caller has
+// it already.
 template <typename T, bool EXT = true, bool QUIET = false>
 __device__ __forceinline__ void cell_field_nb(const FieldArgs<T>& a, long long i, const Region<T>& R,
                                               const v3<T>& m, const v3<T>* nbv, const bool* nbp, const T* cnb,
                                               bool use_hd, const v3<T>& hdv, long long step, v3<T>& H, v3<T>& k,
-                                              bool want_k, bool as_omega = false) {
+                                              bool want_k, bool as_omega = false, const v3<T>* th = nullptr) {
     const long long N = a.N;
     H = mk3<T>(0, 0, 0);
     k = mk3<T>(0, 0, 0);
@@ -248,7 +249,9 @@ __device__ __forceinline__ void cell_field_nb(const FieldArgs<T>& a, long long i
         else if (a.Hd) H = H + ld3(a.Hd, N, i);
     }
     if (!QUIET && (a.terms & MM_TERM_THERMAL) && a.th_scale != (T)0) {
-        if (a.noise && (a.mode == MODE_HEUN2 || a.mode == MODE_DM2)) {
+        if (th) {
+            H = H + *th;
+        } else if (a.noise && (a.mode == MODE_HEUN2 || a.mode == MODE_DM2)) {
             H = H + ld3(a.noise, N, i);
         } else {
             const v3<T> th = thermal_h<T>(a, i, R, step);

@@ -94,11 +94,23 @@ __global__ void __launch_bounds__(kC2RThreads, 3) c2r_field_kernel(FieldArgs<flo
     if (a.gate && !a.st->active) return;
     float* sH = reinterpret_cast<float*>(smem_raw);   // [rpc][3][nx], once the lines are in registers
     const int nx = a.nx, rpc = s.rpc, nrows = a.ny * a.nz;
-    const int row0 = blockIdx.x * rpc;
-    if ((int)threadIdx.x < field_x_fft(G, rpc)) {
-        const int task = threadIdx.x / G, rl = task / 3, comp = task - 3 * rl, row = row0 + rl;
-        const bool valid = rl < rpc && row < nrows;
-        const int z = valid ? row / a.ny : 0, y = valid ? row - z * a.ny : 0;
+    const int row0 = blockIdx.x * rpc, tpr = nx / V, fft = field_x_fft(G, rpc);
+    constexpr bool EXT = KIND == FX_EXT;
+    VecIn<V> in;
+    auto cells = [&](int c, int& rl, int& x0, int& y, int& z) {   // the c-th V cells; false past the grid
+        rl = c / tpr;
+        x0 = V * (c - rl * tpr);
+        z = (row0 + rl) / a.ny;
+        y = row0 + rl - z * a.ny;
+        return row0 + rl < nrows;
+    };
+    int rl, x0, y, z;
+    if ((int)threadIdx.x < fft) {
+        const int task = threadIdx.x / G, comp = task % 3, row = row0 + task / 3;
+        const bool valid = task / 3 < rpc && row < nrows;
+        rl = task / 3;
+        z = valid ? row / a.ny : 0;
+        y = valid ? row - z * a.ny : 0;
         const float2* X = s.spec + ((long long)(comp * a.nz + z) * s.PyA + y) * s.Wk;
         lcx<float>* line = reinterpret_cast<lcx<float>*>(smem_raw) + task * S::LINE;
         float* dst = sH + (rl * 3 + comp) * nx;
@@ -106,19 +118,18 @@ __global__ void __launch_bounds__(kC2RThreads, 3) c2r_field_kernel(FieldArgs<flo
             if (valid && 2 * n < nx) *reinterpret_cast<float2*>(dst + 2 * n) = v;
         });
     } else {
+        // threads without a row: their first cells meanwhile
+        if (!QUIET && (int)threadIdx.x < rpc * tpr && cells(threadIdx.x, rl, x0, y, z))
+            field_vec_load<V, EXT, QUIET>(a, x0, y, z, in);
         if (!S::WARP) __syncthreads();                // (the rows' own exchange)
         __syncthreads();
     }
     __syncthreads();
-    const int tpr = nx / V;
-    for (int c = threadIdx.x; c < rpc * tpr; c += blockDim.x) {
-        const int rl = c / tpr, x0 = V * (c - rl * tpr);
-        const int row = row0 + rl;
-        if (row < nrows) {
-            const int z = row / a.ny, y = row - z * a.ny;
-            field_vec_cells<V, KIND == FX_EXT, true, QUIET>(a, x0, y, z, sH + rl * 3 * nx + x0, nx);
+    for (int c = threadIdx.x; c < rpc * tpr; c += blockDim.x)
+        if (cells(c, rl, x0, y, z)) {
+            if (QUIET || c != (int)threadIdx.x || (int)threadIdx.x < fft) field_vec_load<V, EXT, QUIET>(a, x0, y, z, in);
+            field_vec_finish<V, EXT, true, QUIET>(a, x0, y, z, in, sH + rl * 3 * nx + x0, nx);
         }
-    }
     if (!QUIET && a.tick) fixed_finish(const_cast<DevState*>(a.st), a.tick);
 }
 

@@ -52,8 +52,8 @@ template <> __device__ __forceinline__ const double* err_coef<double>(const DevS
 
 // m_s = m0 + sum_j (dt a_sj) k_j, S = stage index (compile time)
 template <typename T, int S>
-__global__ void __launch_bounds__(256) combine_kernel(const DevState* __restrict__ st, T* const* __restrict__ kptr,
-                                                      const T* __restrict__ m0, T* __restrict__ ms, long long n3) {
+__global__ void __launch_bounds__(256) combine_kernel(const DevState* st, T* const* kptr, const T* m0, T* ms,
+                                                      long long n3) {
     dep_wait();
     if (!st->active) return;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -64,29 +64,27 @@ __global__ void __launch_bounds__(256) combine_kernel(const DevState* __restrict
 #pragma unroll
     for (int j = 0; j < S; ++j) {
         if (j == 1 && S == 6) continue;             // a_7,2 = 0
-        acc += cf[j] * __ldg(&kptr[kslot_of(j, kf)][i]);
+        acc += cf[j] * kptr[kslot_of(j, kf)][i];
     }
     ms[i] = acc;
 }
 
 // FP32, 3N a multiple of 4: four elements per thread as 16-byte vectors.
 template <int S>
-__global__ void __launch_bounds__(256) combine_vec4_kernel(const DevState* __restrict__ st,
-                                                           float* const* __restrict__ kptr,
-                                                           const float* __restrict__ m0, float* __restrict__ ms,
-                                                           long long n4) {
+__global__ void __launch_bounds__(256) combine_vec4_kernel(const DevState* st, float* const* kptr, const float* m0,
+                                                           float* ms, long long n4) {
     dep_wait();
     if (!st->active) return;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n4) return;
     const int kf = st->k_first;
     const float* cf = st->cf32[S];
-    float4 acc = __ldg(reinterpret_cast<const float4*>(m0) + i);
+    float4 acc = reinterpret_cast<const float4*>(m0)[i];
 #pragma unroll
     for (int j = 0; j < S; ++j) {
         if (j == 1 && S == 6) continue;             // a_7,2 = 0
         const float c = cf[j];
-        const float4 k = __ldg(reinterpret_cast<const float4*>(kptr[kslot_of(j, kf)]) + i);
+        const float4 k = reinterpret_cast<const float4*>(kptr[kslot_of(j, kf)])[i];
         acc.x += c * k.x; acc.y += c * k.y; acc.z += c * k.z; acc.w += c * k.w;
     }
     reinterpret_cast<float4*>(ms)[i] = acc;
@@ -94,7 +92,7 @@ __global__ void __launch_bounds__(256) combine_vec4_kernel(const DevState* __res
 
 // per-cell error |dt sum e_j k_j|, block max, atomic max into st->err(_f)
 template <typename T>
-__global__ void error_kernel(DevState* st, T* const* __restrict__ kptr, long long N) {
+__global__ void error_kernel(DevState* st, T* const* kptr, long long N) {
     dep_wait();
     if (!st->active) return;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -194,8 +192,7 @@ __global__ void controller_kernel(DevState* st, int prec) {
 }
 
 template <typename T>
-__global__ void accept_kernel(const DevState* __restrict__ st, const T* __restrict__ m5, T* __restrict__ m0,
-                              long long N) {
+__global__ void accept_kernel(const DevState* st, const T* m5, T* m0, long long N) {
     dep_wait();
     if (!st->active || !st->accept) return;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -348,22 +345,19 @@ void heun_batch_advance(mm_ctx* c) {
 // m0 + c dt k with c = 1/2, 1/2, 1, then m0 <- normalise(m0 + dt/6 (k1 +
 // 2 k2 + 2 k3 + k4)); dt from the device state (fixed per context).
 template <typename T>
-__global__ void __launch_bounds__(256) rk4_stage_kernel(const DevState* __restrict__ st, const T* __restrict__ m0,
-                                                        const T* __restrict__ k, double c, T* __restrict__ out,
+__global__ void __launch_bounds__(256) rk4_stage_kernel(const DevState* st, const T* m0, const T* k, double c, T* out,
                                                         long long n3) {
     dep_wait();
     if (!st->active) return;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n3) return;
     const T h = (T)(c * st->dt);
-    out[i] = m0[i] + h * __ldg(k + i);
+    out[i] = m0[i] + h * k[i];
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) rk4_final_kernel(DevState* st, T* __restrict__ m0,
-                                                        const T* __restrict__ k1, const T* __restrict__ k2,
-                                                        const T* __restrict__ k3, const T* __restrict__ k4,
-                                                        long long N, unsigned* tick) {
+__global__ void __launch_bounds__(256) rk4_final_kernel(DevState* st, T* m0, const T* k1, const T* k2, const T* k3,
+                                                        const T* k4, long long N, unsigned* tick) {
     dep_wait();
     if (!st->active) return;
     const T h6 = (T)(st->dt / 6.0);
@@ -436,7 +430,7 @@ void dm_step(mm_ctx* c) {
 // Adaptive Depondt-Mertens: err = max over cells |cand - m*| (the corrector
 // against the first-order predictor), block max, atomic max into st->err(_f).
 template <typename T>
-__global__ void dm_error_kernel(DevState* st, const T* __restrict__ cand, const T* __restrict__ mstar, long long N) {
+__global__ void dm_error_kernel(DevState* st, const T* cand, const T* mstar, long long N) {
     dep_wait();
     if (!st->active) return;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;

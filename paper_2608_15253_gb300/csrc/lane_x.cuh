@@ -73,7 +73,7 @@ __device__ __forceinline__ void x_stage_pairs(const XLaneArgs<T>& a, long long g
     auto slot = [&](int s) { return reinterpret_cast<const cplx<T>*>(s == 0 ? (kf ? a.k[6] : a.k[0]) : a.k[s]) + o; };
 #pragma unroll
     for (int q = 0; q < QIN; ++q)
-        x[q] = q * G + t < nin ? __ldg(reinterpret_cast<const cplx<T>*>(a.m0) + o + q * G + t) : mkc<T>(0, 0);
+        x[q] = q * G + t < nin ? reinterpret_cast<const cplx<T>*>(a.m0)[o + q * G + t] : mkc<T>(0, 0);
 #pragma unroll 1
     for (int s = 0; s < a.stage; s += 2) {
         const bool two = s + 1 < a.stage && !(s == 0 && a.stage == 6);   // a_7,2 = 0
@@ -81,9 +81,9 @@ __device__ __forceinline__ void x_stage_pairs(const XLaneArgs<T>& a, long long g
         const cplx<T>*k0 = slot(s), *k1 = two ? slot(s + 1) : k0;
         cplx<T> d0[QIN], d1[QIN];
 #pragma unroll
-        for (int q = 0; q < QIN; ++q) d0[q] = q * G + t < nin ? __ldg(k0 + q * G + t) : mkc<T>(0, 0);
+        for (int q = 0; q < QIN; ++q) d0[q] = q * G + t < nin ? k0[q * G + t] : mkc<T>(0, 0);
 #pragma unroll
-        for (int q = 0; q < QIN; ++q) d1[q] = two && q * G + t < nin ? __ldg(k1 + q * G + t) : mkc<T>(0, 0);
+        for (int q = 0; q < QIN; ++q) d1[q] = two && q * G + t < nin ? k1[q * G + t] : mkc<T>(0, 0);
 #pragma unroll
         for (int q = 0; q < QIN; ++q) {
             x[q].x = x[q].x + c0 * d0[q].x;
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(G* ROWS) lane_r2c_kernel(XLaneArgs<T> a) {
         } else {
 #pragma unroll
             for (int q = 0; q < S::QIN; ++q)
-                x[q] = q * G + t < nin ? __ldg(reinterpret_cast<const cplx<T>*>(a.in + g0) + q * G + t) : mkc<T>(0, 0);
+                x[q] = q * G + t < nin ? reinterpret_cast<const cplx<T>*>(a.in + g0)[q * G + t] : mkc<T>(0, 0);
         }
 #pragma unroll
         for (int q = 0; q < S::QIN; ++q) v[q] = {x[q].x * a.ms, x[q].y * a.ms};
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(G* ROWS) lane_r2c_kernel(XLaneArgs<T> a) {
                 const cplx<T>* p = reinterpret_cast<const cplx<T>*>(src + g0);
 #pragma unroll
                 for (int q = 0; q < S::QIN; ++q) {
-                    const cplx<T> d = q * G + t < nin ? __ldg(p + q * G + t) : mkc<T>(0, 0);
+                    const cplx<T> d = q * G + t < nin ? p[q * G + t] : mkc<T>(0, 0);
                     x[2 * q] = first ? d.x : x[2 * q] + c * d.x;
                     x[2 * q + 1] = first ? d.y : x[2 * q + 1] + c * d.y;
                 }
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(G* ROWS) lane_r2c_kernel(XLaneArgs<T> a) {
 #pragma unroll
                 for (int q = 0; q < 2 * S::QIN; ++q) {
                     const int n = 2 * ((q / 2) * G + t) + q % 2;
-                    const T d = n < a.nx ? __ldg(src + g0 + n) : (T)0;
+                    const T d = n < a.nx ? src[g0 + n] : (T)0;
                     x[q] = first ? d : x[q] + c * d;
                 }
             }
@@ -426,14 +426,14 @@ __global__ void __launch_bounds__(128) fine_r2c_kernel(XLaneArgs<T> a) {
             T k[6];
 #pragma unroll
             for (int s = 0; s < 6; ++s)
-                k[s] = s < a.stage && !(s == 1 && a.stage == 6) ? __ldg((s == 0 ? (kf ? a.k[6] : a.k[0]) : a.k[s]) + e) : (T)0;
-            x = __ldg(a.m0 + e);
+                k[s] = s < a.stage && !(s == 1 && a.stage == 6) ? (s == 0 ? (kf ? a.k[6] : a.k[0]) : a.k[s])[e] : (T)0;
+            x = a.m0[e];
 #pragma unroll
             for (int s = 0; s < 6; ++s)
                 if (s < a.stage && !(s == 1 && a.stage == 6)) x += cf[s] * k[s];
             a.ms_out[e] = x;
         } else {
-            x = __ldg(a.in + e);
+            x = a.in[e];
         }
         return rg ? x * __ldg(&a.lut[rg[n]].Ms) : x * a.ms;
     };

@@ -3,7 +3,10 @@
 // in dep_wait() (common.cuh) until that has finished and its writes are
 // visible.  Captured into a graph the edge stays programmatic.  Only for
 // kernels that call dep_wait() before their first access to data of earlier
-// kernels.
+// kernels, and that read such data with plain loads: __ldg, and a const
+// __restrict__ pointer, which lets the compiler make one of a load, are for
+// data that is constant from the kernel's launch on, here the tables filled at
+// setup (twiddles, tensor, materials), and may be moved above the wait.
 #pragma once
 
 #include <cuda_runtime.h>
