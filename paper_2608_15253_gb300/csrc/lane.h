@@ -27,6 +27,7 @@ template <typename T> LaneKern<T> lane_col(int L, bool forward);    // Y passes 
 
 template <> LaneKern<float> lane_conv3<float>(int L);
 template <> LaneKern<double> lane_conv3<double>(int L);
+LaneKern<float> lane_conv3_long(int L);                         // its lines of 162 points and more
 template <> LaneKern<float> lane_film<float>(int L);
 template <> LaneKern<double> lane_film<double>(int L);
 template <> LaneKern<float> lane_films<float>(int L);

@@ -30,7 +30,7 @@ template <> LaneKern<float> lane_conv3<float>(int L) {
         MM_CONV3_F(MM_CASE)
 #undef MM_CASE
         case 128: return {lane_conv_kernel<float2, 128, 8, 16, 8, 3, true, 2, true>, 192, 16, lane_conv_smem<float2, 128, 8, 16, 8, 6, true>(), true};
-        default: return {};
+        default: return lane_conv3_long(L);
     }
 }
 
