@@ -31,6 +31,21 @@ def _pass_us(mm, shape, name, integrator="rk4"):
         mm.mm_destroy(ctx)
 
 
+@pytest.mark.parametrize("prec", [64, 32])
+@pytest.mark.parametrize("ny", [7, 8])
+@pytest.mark.parametrize("nx", [3, 64])
+def test_short_y_lines(nx, ny, prec):
+    _check(W.Grid(nx, ny, 5, 2e-9, 2e-9, 2e-9), prec)
+
+
+@pytest.mark.parametrize("name", ["fft_y_fwd", "fft_y_inv"])
+def test_short_y_lines_have_a_kernel(name):
+    """Eight rows (16 points) against sixteen (32 points), in half of a pass's
+    columns: launches alone, the same kernel."""
+    mm = need_gpu()
+    assert _pass_us(mm, (64, 8, 6), name) < 1.5 * _pass_us(mm, (64, 16, 6), name)
+
+
 LONG_Z = [162, 192, 216, 256, 324, 432, 512, 1024]
 
 
