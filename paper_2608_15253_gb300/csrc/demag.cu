@@ -780,10 +780,10 @@ static bool launch_lane_y(mm_ctx* c, bool fwd, cplx<T>* S, const char* name, dou
 template <typename T>
 static bool launch_lane_z(mm_ctx* c, cplx<T>* S, double bytes) {
     const DemagPlan& d = c->dm;
-    const LaneKern<T> k = lane_conv3<T>(d.Pz);
+    const long long plane = (long long)d.Py * d.Wk, Ky = d.Py / 2 + 1, Kz = d.Pz / 2 + 1;
+    const LaneKern<T> k = lane_conv3<T>(d.Pz, (int)(Ky * d.Wk));
     if (!k.kern) return false;
     LaneArgs<T> a{};
-    const long long plane = (long long)d.Py * d.Wk, Ky = d.Py / 2 + 1, Kz = d.Pz / 2 + 1;
     a.base = S;
     a.comp_stride = c->grid.nz * plane;
     a.line_stride = plane;
@@ -851,7 +851,7 @@ template <typename T>
 static cudaError_t lane_attributes(const DemagPlan& d, bool three_d) {
     const LaneKern<T> ks[] = {three_d ? lane_col<T>(d.Py, true) : lane_film<T>(d.Py),
                               three_d ? lane_col<T>(d.Py, false) : lane_films<T>(d.Py),
-                              three_d ? lane_conv3<T>(d.Pz) : LaneKern<T>{}};
+                              three_d ? lane_conv3<T>(d.Pz, (d.Py / 2 + 1) * d.Wk) : LaneKern<T>{}};
     for (const LaneKern<T>& k : ks)
         if (k.kern) {
             const cudaError_t e = cudaFuncSetAttribute(k.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);

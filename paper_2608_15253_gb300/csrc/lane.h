@@ -20,14 +20,14 @@ struct LaneKern {
     bool persistent = false;        // CTAs loop over the column tiles
 };
 
-template <typename T> LaneKern<T> lane_conv3(int L);            // middle pass of a 3-D grid
+template <typename T> LaneKern<T> lane_conv3(int L, int columns);   // middle pass of a 3-D grid, columns of one side
 template <typename T> LaneKern<T> lane_film(int L);             // middle pass of one film
 template <typename T> LaneKern<T> lane_films(int L);            // middle pass of many films
 template <typename T> LaneKern<T> lane_col(int L, bool forward);    // Y passes of a 3-D grid
 
-template <> LaneKern<float> lane_conv3<float>(int L);
-template <> LaneKern<double> lane_conv3<double>(int L);
-LaneKern<float> lane_conv3_long(int L);                         // its lines of 162 points and more
+template <> LaneKern<float> lane_conv3<float>(int L, int columns);
+template <> LaneKern<double> lane_conv3<double>(int L, int columns);
+LaneKern<float> lane_conv3_long(int L, int columns);            // its lines of 162 points and more
 template <> LaneKern<float> lane_film<float>(int L);
 template <> LaneKern<double> lane_film<double>(int L);
 template <> LaneKern<float> lane_films<float>(int L);

@@ -23,18 +23,18 @@ namespace mm {
     X(18, 2, 9, 16, 1) X(24, 3, 8, 16, 1) X(27, 3, 9, 16, 1) X(32, 4, 8, 16, 1) X(36, 4, 9, 16, 1) X(48, 6, 8, 8, 1) \
     X(54, 6, 9, 8, 1) X(64, 8, 8, 8, 1) X(72, 8, 9, 8, 1) X(81, 9, 9, 8, 1) X(96, 8, 12, 8, 1) X(128, 8, 16, 8, 1)
 
-template <> LaneKern<float> lane_conv3<float>(int L) {
+template <> LaneKern<float> lane_conv3<float>(int L, int columns) {
     switch (L) {
 #define MM_CASE(l, g, q, tp, mb) \
     case l: return {lane_conv_kernel<float, l, g, q, tp, 1, true, mb, false>, g * tp, tp, lane_conv_smem<float, l, g, q, tp, 6, false>(), false};
         MM_CONV3_F(MM_CASE)
 #undef MM_CASE
         case 128: return {lane_conv_kernel<float2, 128, 8, 16, 8, 3, true, 2, true>, 192, 16, lane_conv_smem<float2, 128, 8, 16, 8, 6, true>(), true};
-        default: return lane_conv3_long(L);
+        default: return lane_conv3_long(L, columns);
     }
 }
 
-template <> LaneKern<double> lane_conv3<double>(int L) {
+template <> LaneKern<double> lane_conv3<double>(int L, int) {
     switch (L) {
 #define MM_CASE(l, g, q, tp, mb) \
     case l: return {lane_conv_kernel<double, l, g, q, tp, 1, true, mb, false>, g * tp, tp, lane_conv_smem<double, l, g, q, tp, 6, false>(), false};

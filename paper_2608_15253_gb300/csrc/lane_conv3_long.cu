@@ -21,15 +21,22 @@ namespace mm {
 #define MM_CONV3_LONG(X) \
     X(162, 9, 18, 8, 3, 1, true) X(192, 12, 16, 16, 3, 1, true) X(216, 12, 18, 16, 3, 1, true) X(256, 16, 16, 8, 1, 2, false) \
     X(324, 18, 18, 8, 1, 2, false) X(432, 16, 27, 8, 3, 1, false) X(512, 16, 32, 8, 3, 1, false) X(1024, 16, 64, 4, 3, 1, false)
+// Where persistent CTAs of 16 columns do not reach half of the SMs: 8 columns and
+// one side each, four times as many (L = 192 / 216, 8x8 columns 15.9 / 18.1 -> 9.9 / 12.0 us, 32x32 16.0 / 18.2 -> 12.0 / 14.1).
+#define MM_CONV3_FEW(X) X(192, 12, 16, 8, 3, 3, false) X(216, 12, 18, 8, 3, 3, false)
 
-LaneKern<float> lane_conv3_long(int L) {
-    switch (L) {
+LaneKern<float> lane_conv3_long(int L, int columns) {
 #define MM_CASE(l, g, q, tp, cs, mb, st) \
     case l: return {lane_conv_kernel<float, l, g, q, tp, cs, true, mb, st>, cs * g * tp, tp, lane_conv_smem<float, l, g, q, tp, 6, st>(), st};
+    if (columns <= 8 * sm_count()) switch (L) {
+        MM_CONV3_FEW(MM_CASE)
+        default: break;
+    }
+    switch (L) {
         MM_CONV3_LONG(MM_CASE)
-#undef MM_CASE
         default: return {};
     }
+#undef MM_CASE
 }
 
 }  // namespace mm

@@ -55,6 +55,13 @@ def test_long_z_lines(L):
         _check(W.Grid(9, 6, nz, 3e-9, 3e-9, 3e-9), 32)
 
 
+@pytest.mark.parametrize("L", [162, 192, 216])
+def test_long_z_lines_of_many_columns(L):
+    """(few and many columns have kernels of their own at 192 and 216 points)"""
+    for nz in _sizes(L):
+        _check(W.Grid(40, 62, nz, 3e-9, 3e-9, 3e-9), 32)
+
+
 @pytest.mark.parametrize("L", LONG_Z)
 def test_long_z_lines_have_a_kernel(L):
     mm = need_gpu()
