@@ -39,6 +39,9 @@ template <> LaneKern<double> lane_col<double>(int L, bool forward);
 // per row, at most `rows` rows per CTA.
 template <typename T> struct XLaneArgs;
 
+// FP32 rows of half length 1024, for the separate X passes alone
+#define MM_XLANE_LONG(X) X(1024, 16, 64, 4)
+
 template <typename T>
 struct XLane {
     void (*r2c[3])(XLaneArgs<T>) = {};          // by XInput: plain rows, stage state, anything

@@ -46,6 +46,53 @@ def test_short_y_lines_have_a_kernel(name):
     assert _pass_us(mm, (64, 8, 6), name) < 1.5 * _pass_us(mm, (64, 16, 6), name)
 
 
+@pytest.mark.parametrize("cells", [False, True])
+@pytest.mark.parametrize("nx", [973, 1023, 1024])
+def test_long_rows(nx, cells):
+    """The smallest, the largest odd and the largest row of half length 1024."""
+    mm = need_gpu()
+    from oracle.demag import demag_spectrum, h_demag
+    from gpu_util import TERMS, oracle_problem, rel_err
+    grid = W.Grid(nx, 3, 1, 2e-9, 2e-9, 1e-9)
+    mat = W.with_cells(MAT, W.random_material_cells(grid, nx)) if cells else MAT
+    ctx = make_ctx(mm, grid, mat, precision=32)
+    try:
+        mm.mm_set_m(ctx, 0, W.m_random_sphere(grid, seed=nx))
+        m = mm.mm_get_m(ctx, 0, (3,) + grid.shape)
+        p = oracle_problem(grid, mat)
+        ref = np.where(p.present, h_demag(m, p, demag_spectrum(p.shape, p.d)), 0.0)
+        assert rel_err(mm.mm_get_heff(ctx, 0, m.shape, TERMS["demag"]), ref) < 5e-6
+    finally:
+        mm.mm_destroy(ctx)
+
+
+@pytest.mark.parametrize("shape", [(1024, 5, 1), (975, 3, 2)])
+def test_stage_state_of_long_rows(shape):
+    """Ten RK45 steps replayed from the oracle."""
+    mm = need_gpu()
+    from gpu_util import oracle_problem
+    from oracle.llg import Solver
+    grid = W.Grid(*shape, 2e-9, 2e-9, 2e-9)
+    m0 = W.m_random_sphere(grid, seed=7)
+    o = Solver(oracle_problem(grid, MAT), m0, dt=1e-14, rtol=1e-6)
+    dts = [o.rk45_step() for _ in range(10)]
+    ctx = make_ctx(mm, grid, MAT, precision=32, dt=1e-14, rtol=1e-6)
+    try:
+        mm.mm_set_m(ctx, 0, m0)
+        mm.mm_step_dt(ctx, dts)
+        assert np.abs(mm.mm_get_m(ctx, 0, m0.shape) - o.m).max() <= 1e-5
+    finally:
+        mm.mm_destroy(ctx)
+
+
+@pytest.mark.parametrize("name", ["fft_x_r2c", "fft_x_c2r"])
+def test_long_rows_have_a_kernel(name):
+    """Rows of 1024 cells against rows of 512 in as many rows: twice the work."""
+    mm = need_gpu()
+    scale = _pass_us(mm, (511, 600, 1), name)       # (odd: the inverse pass is a launch of its own)
+    assert _pass_us(mm, (1023, 600, 1), name) < 3 * scale
+
+
 LONG_Z = [162, 192, 216, 256, 324, 432, 512, 1024]
 
 
