@@ -243,7 +243,7 @@ static void free_all(mm_ctx* c) {
     c->batch = nullptr;
     surrogate_free(c);
     void* bufs[] = {c->d_region, c->d_lut, c->d_cpair, c->d_m, c->d_mtmp, c->d_kslot, c->d_hd, c->d_hbuf,
-                    c->d_bcell, c->d_state, c->d_replay, c->d_red, c->d_stage, c->d_strain, c->d_flag, c->d_tick};
+                    c->d_bcell, c->d_state, c->d_replay, c->d_red, c->d_stage, c->d_strain, c->d_flag};
     for (void* b : bufs) cudaFree(b);
     for (auto& k : c->d_k) cudaFree(k);
     if (c->own_stream) cudaStreamDestroy(c->own_stream);
@@ -422,8 +422,6 @@ mm_status mm_create(const mm_grid* grid, const mm_material* mat, const mm_config
     c->red_cap = 2 * 304 + 32;
     TRY(alloc(c, (void**)&c->d_red, sizeof(double) * c->red_cap, "reduction partials"));
     TRY(alloc(c, (void**)&c->d_flag, sizeof(int), "state flag"));
-    TRY(alloc(c, (void**)&c->d_tick, sizeof(unsigned), "block counter"));
-    cudaMemset(c->d_tick, 0, sizeof(unsigned));
     if (c->terms & MM_TERM_DEMAG) {
         TRY(alloc(c, &c->d_hd, vb, "demag field"));
         TRY(demag_setup(c));
@@ -554,8 +552,6 @@ mm_status mm_create_batch(int R, const mm_grid* grids, const mm_material* mat, c
     c->red_cap = 2 * 304 + 32;
     TRY(alloc(c, (void**)&c->d_red, sizeof(double) * c->red_cap, "reduction partials"));
     TRY(alloc(c, (void**)&c->d_flag, sizeof(int), "state flag"));
-    TRY(alloc(c, (void**)&c->d_tick, sizeof(unsigned), "block counter"));
-    cudaMemset(c->d_tick, 0, sizeof(unsigned));
     c->batch = batch_new();
     TRY(batch_setup(c, c->batch, c->rgrid, c->rkey, (c->terms & MM_TERM_DEMAG) != 0));
     TRY(batch_upload(c, c->batch, c->rT, c->rJ));

@@ -68,18 +68,6 @@ __device__ __forceinline__ double warp_max(double v) {
 // 2.50 -> 3.44 ms, 128x32 FP64 3.79 -> 3.69 ms).
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// True in the one thread that calls it last over the grid, one call per block
-// (every block of the launch must call it); resets the counter for the next
-// launch.  What it reads from other blocks has to bypass L1 (__ldcg).
-__device__ __forceinline__ bool last_block(unsigned* tick) {
-    __threadfence();
-    const unsigned n = gridDim.x * gridDim.y * gridDim.z;
-    if (atomicAdd(tick, 1u) + 1u != n) return false;
-    *tick = 0;
-    __threadfence();
-    return true;
-}
-
 // Neumaier-compensated FP64 sum: value = s + c.
 struct CompSum {
     double s, c;

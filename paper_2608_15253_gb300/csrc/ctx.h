@@ -157,7 +157,6 @@ struct mm_ctx {
     size_t replay_cap = 0;
     double* d_red = nullptr;    // reduction partials
     int* d_flag = nullptr;      // one device int (mm_set_m: did the state change)
-    unsigned* d_tick = nullptr; // block counter of the kernels whose last block does the step's bookkeeping
     size_t red_cap = 0;
 
     mm::DemagPlan dm;
@@ -225,14 +224,14 @@ mm_status newell_gpu(long count, const int* ijk, double dx, double dy, double dz
 enum FieldMode { MODE_H = 0, MODE_K = 1, MODE_HEUN1 = 2, MODE_HEUN2 = 3, MODE_DM1 = 4, MODE_DM2 = 5 };
 void field_launch(mm_ctx* c, int mode, unsigned terms, const void* m, const void* Hd,
                   void* out, void* out2, const void* m0, const void* k1, long long step_override,
-                  int gate, int kstage, bool finish = false);
+                  int gate, int kstage);
 void thermal_raw_launch(mm_ctx* c, long long step, uint32_t* d_raw, void* d_h);
 // inverse X pass + field kernel in one launch (the demag spectrum of the
 // state must be ready); field_c2r_fusable says whether the grid allows it
 bool field_c2r_fusable(const mm_ctx* c, int mode, unsigned terms);
 cudaError_t field_c2r_setup(const mm_ctx* c);
 void field_c2r_launch(mm_ctx* c, int mode, unsigned terms, const void* m, void* out, void* out2, const void* m0,
-                      const void* k1, long long step_override, int gate, int kstage, bool finish = false);
+                      const void* k1, long long step_override, int gate, int kstage);
 
 // batch.cu
 BatchHost* batch_new();
@@ -275,8 +274,8 @@ void demag_eval(mm_ctx* c, const void* m, void* Hd);   // exact or surrogate
 void heun_batch_begin(mm_ctx* c);
 void heun_batch_advance(mm_ctx* c);
 void rk45_first_slope(mm_ctx* c);          // k1 = f(m0) into the FSAL slot
-// Begins the first fixed step of a request on the device; the last block of a
-// step's last kernel begins the next one.
+// Begins the first fixed step of a request on the device; the end of a step
+// begins the next one.
 void step_begin(mm_ctx* c);
 void rk45_attempt(mm_ctx* c);               // one attempted DOPRI5 step
 void heun_step(mm_ctx* c);

@@ -26,7 +26,6 @@ __global__ void __launch_bounds__(256) field_kernel(FieldArgs<T> a) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x < a.nx && y < a.ny) field_cell<T, UNIF, EXT>(a, x, y, blockIdx.z);
-    if (a.tick) fixed_finish(const_cast<DevState*>(a.st), a.tick);
 }
 
 template <int V, bool EXT, bool QUIET = false>
@@ -40,7 +39,6 @@ __global__ void __launch_bounds__(256) field_vec_kernel(FieldArgs<float> a) {
         field_vec_load<V, EXT, QUIET>(a, x0, y, blockIdx.z, in);
         field_vec_finish<V, EXT, false, QUIET>(a, x0, y, blockIdx.z, in, nullptr, 0);
     }
-    if (!QUIET && a.tick) fixed_finish(const_cast<DevState*>(a.st), a.tick);
 }
 
 constexpr int kFieldV = 4;   // cells per thread of the one-material FP32 kernel (4 measured faster than 2)
@@ -130,9 +128,8 @@ static const char* const kFieldNames[6] = {"field_H", "field_k", "field_heun1", 
 
 template <typename T>
 static void field_launch_t(mm_ctx* c, int mode, unsigned terms, const T* m, const T* Hd, T* out, T* out2,
-                           const T* m0, const T* k1, long long step_override, int gate, int kstage, bool finish) {
+                           const T* m0, const T* k1, long long step_override, int gate, int kstage) {
     FieldArgs<T> a = field_args<T>(c, mode, terms, m, Hd, out, out2, m0, k1, step_override, gate, kstage);
-    if (finish) a.tick = c->d_tick;
     const mm_grid& g = c->grid;
     // rows of 32 cells per warp, eight warps to a CTA; on small grids fewer, so
     // that every scheduler gets a warp (FP64, 128x32: 15.4 -> 10.7 us; 16 CTAs of
@@ -163,13 +160,13 @@ static void field_launch_t(mm_ctx* c, int mode, unsigned terms, const T* m, cons
 }
 
 void field_launch(mm_ctx* c, int mode, unsigned terms, const void* m, const void* Hd, void* out, void* out2,
-                  const void* m0, const void* k1, long long step_override, int gate, int kstage, bool finish) {
+                  const void* m0, const void* k1, long long step_override, int gate, int kstage) {
     if (c->prec == 32)
         field_launch_t<float>(c, mode, terms, (const float*)m, (const float*)Hd, (float*)out, (float*)out2,
-                              (const float*)m0, (const float*)k1, step_override, gate, kstage, finish);
+                              (const float*)m0, (const float*)k1, step_override, gate, kstage);
     else
         field_launch_t<double>(c, mode, terms, (const double*)m, (const double*)Hd, (double*)out, (double*)out2,
-                               (const double*)m0, (const double*)k1, step_override, gate, kstage, finish);
+                               (const double*)m0, (const double*)k1, step_override, gate, kstage);
 }
 
 // Inverse X pass + field kernel in one launch (FP32, one material, even nx,
@@ -222,14 +219,13 @@ static void fine_field_launch(mm_ctx* c, int mode, unsigned terms, const double*
 }
 
 void field_c2r_launch(mm_ctx* c, int mode, unsigned terms, const void* m, void* out, void* out2, const void* m0,
-                      const void* k1, long long step_override, int gate, int kstage, bool finish) {
+                      const void* k1, long long step_override, int gate, int kstage) {
     if (c->prec == 64) {
         fine_field_launch(c, mode, terms, (const double*)m, (double*)out, step_override, gate, kstage);
         return;
     }
     FieldArgs<float> a = field_args<float>(c, mode, terms, (const float*)m, nullptr, (float*)out, (float*)out2,
                                            (const float*)m0, (const float*)k1, step_override, gate, kstage);
-    if (finish) a.tick = c->d_tick;
     const DemagPlan& d = c->dm;
     const int nx = c->grid.nx;
     const long long rows = (long long)c->grid.ny * c->grid.nz;

@@ -80,7 +80,6 @@ struct FieldArgs {
     const DevState* st;   // step counter, dt, active flag
     int gate;             // 1: skip the launch when st->active == 0
     long long step_override;  // >= 0: use this step for the noise
-    unsigned* tick;       // not null: this launch ends a fixed step (its last block advances the state)
     T* const* kptr;       // MODE_K with out == null: write to the FSAL slot of stage kstage
     int kstage;           // 0 (k1) or 6 (k7)
     // torques
@@ -98,25 +97,6 @@ struct FieldArgs {
     int rk1, rk2;         // RKKY layers
     T rkky_c;             // J / dz (times 1/(mu0 Ms) -> A/m per unit m)
 };
-
-// Whether a fixed step follows, and its size.
-__device__ __forceinline__ void fixed_begin(DevState* st) {
-    st->active = (st->accepted < st->target && st->t < st->t_end && st->status == 0) ? 1 : 0;
-    st->dt_eff = st->dt;
-}
-// End of a fixed step in the last block of its last kernel: t += dt, the
-// counters, and the next step begins.  Every block of an active launch calls
-// it with all of its threads.
-__device__ __forceinline__ void fixed_finish(DevState* st, unsigned* tick) {
-    __syncthreads();
-    if (threadIdx.x == 0 && threadIdx.y == 0 && last_block(tick)) {
-        st->t += st->dt;
-        st->step += 1;
-        st->accepted += 1;
-        st->attempts += 1;
-        fixed_begin(st);
-    }
-}
 
 // Thermal field of cell i at noise counter `step`: Philox4x32-10 keyed by
 // (key0, key1) on the counter (i, step), Box-Muller, times

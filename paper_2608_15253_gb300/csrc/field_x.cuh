@@ -130,7 +130,6 @@ __global__ void __launch_bounds__(kC2RThreads, 3) c2r_field_kernel(FieldArgs<flo
             if (QUIET || c != (int)threadIdx.x || (int)threadIdx.x < fft) field_vec_load<V, EXT, QUIET>(a, x0, y, z, in);
             field_vec_finish<V, EXT, true, QUIET>(a, x0, y, z, in, sH + rl * 3 * nx + x0, nx);
         }
-    if (!QUIET && a.tick) fixed_finish(const_cast<DevState*>(a.st), a.tick);
 }
 
 }  // namespace mm

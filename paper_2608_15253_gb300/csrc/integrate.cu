@@ -11,12 +11,10 @@
 // on accept m <- m5/|m5| and k7 becomes k1 (slot rotation, no copy).
 #include <cuda_runtime.h>
 
-#include <algorithm>
 #include <cmath>
 
 #include "common.cuh"
 #include "ctx.h"
-#include "field_dev.cuh"
 #include "launch.h"
 
 namespace mm {
@@ -205,14 +203,10 @@ __global__ void accept_kernel(const DevState* st, const T* m5, T* m0, long long 
     m0[2 * N + i] = z * inv;
 }
 
-// Heun step bookkeeping (fixed dt): t += dt, step += 1.
-__global__ void heun_advance_kernel(DevState* st) {
-    dep_wait();
-    if (!st->active) return;
-    st->t += st->dt;
-    st->step += 1;
-    st->accepted += 1;
-    st->attempts += 1;
+// Whether a fixed step follows, and its size.
+__device__ __forceinline__ void fixed_begin(DevState* st) {
+    st->active = (st->accepted < st->target && st->t < st->t_end && st->status == 0) ? 1 : 0;
+    st->dt_eff = st->dt;
 }
 
 __global__ void heun_begin_kernel(DevState* st) {
@@ -220,22 +214,32 @@ __global__ void heun_begin_kernel(DevState* st) {
     fixed_begin(st);
 }
 
+// End of a fixed step: t += dt, the counters, and the next step begins.  A kernel
+// of one thread, 2 us at most; the same in the last block of the step's last
+// kernel, found by a counter, was no faster on small grids (128x128 to 512x512
+// Heun films equal or 1 % slower) and kept large ones waiting for their writes and
+// the counter (512x512x32 without demag 278 against 255 us a step, 8 to 9 % from
+// 1 M cells on).
+__global__ void fixed_next_kernel(DevState* st) {
+    dep_wait();
+    if (!st->active) return;
+    st->t += st->dt;
+    st->step += 1;
+    st->accepted += 1;
+    st->attempts += 1;
+    fixed_begin(st);
+}
+
 // Fixed steps of a single instance: the first of a request begins here, the
-// others in the last block of the step before (256x256 film at 300 K, 8 -> 6
-// launches a step: 1.70 -> 1.65 ms for 32 steps).  The adaptive schemes keep
-// their one-thread kernels: the same bookkeeping in the last block of the
-// error and accept kernels was no faster (512x512 film 1.53 -> 1.57 ms).
+// others at the end of the step before.
 void step_begin(mm_ctx* c) {
     if (c->batch || c->integrator == MM_RK45 || c->integrator == MM_DM_ADAPTIVE) return;
     LaunchScope ls(c, "step_begin", 0.0);
     launch_dep(heun_begin_kernel, 1, 1, 0, c, c->d_state);
 }
-
-// CTAs of a kernel that counts its blocks: enough to fill the chip, few
-// enough that the counter costs nothing (one atomic per 256 cells cost 50 of
-// 127 us at 512x512x64).
-static unsigned counted_blocks(long long N, unsigned tb) {
-    return (unsigned)std::min<long long>((N + tb - 1) / tb, 152 * 8);
+static void step_next(mm_ctx* c) {
+    LaunchScope ls(c, "step_next", 0.0);
+    launch_dep(fixed_next_kernel, 1, 1, 0, c, c->d_state);
 }
 
 void demag_eval(mm_ctx* c, const void* m, void* Hd) {
@@ -247,14 +251,14 @@ void demag_eval(mm_ctx* c, const void* m, void* Hd) {
 // grid that allows it, the last demag pass (inverse X) runs inside the
 // field kernel and H_demag never goes through global memory.
 static void demag_and_field(mm_ctx* c, bool demag, int mode, unsigned terms, const void* m, void* out, void* out2,
-                            const void* m0, const void* k1, int gate, int kstage, bool finish = false) {
+                            const void* m0, const void* k1, int gate, int kstage) {
     if (demag && !surrogate_active(c) && field_c2r_fusable(c, mode, terms)) {
         demag_apply_partial(c, m, 0);
-        field_c2r_launch(c, mode, terms, m, out, out2, m0, k1, -1, gate, kstage, finish);
+        field_c2r_launch(c, mode, terms, m, out, out2, m0, k1, -1, gate, kstage);
         return;
     }
     if (demag) demag_eval(c, m, c->d_hd);
-    field_launch(c, mode, terms, m, demag ? c->d_hd : nullptr, out, out2, m0, k1, -1, gate, kstage, finish);
+    field_launch(c, mode, terms, m, demag ? c->d_hd : nullptr, out, out2, m0, k1, -1, gate, kstage);
 }
 
 template <typename T>
@@ -338,7 +342,7 @@ void heun_batch_begin(mm_ctx* c) {
 
 void heun_batch_advance(mm_ctx* c) {
     LaunchScope ls(c, "heun_advance", 0.0);
-    launch_dep(heun_advance_kernel, 1, 1, 0, c, c->d_state);
+    launch_dep(fixed_next_kernel, 1, 1, 0, c, c->d_state);
 }
 
 // Classical RK4 (Methods, "Integrators": fixed step): stage states
@@ -356,24 +360,23 @@ __global__ void __launch_bounds__(256) rk4_stage_kernel(const DevState* st, cons
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) rk4_final_kernel(DevState* st, T* m0, const T* k1, const T* k2, const T* k3,
-                                                        const T* k4, long long N, unsigned* tick) {
+__global__ void __launch_bounds__(256) rk4_final_kernel(const DevState* st, T* m0, const T* k1, const T* k2,
+                                                        const T* k3, const T* k4, long long N) {
     dep_wait();
     if (!st->active) return;
+    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (i >= N) return;
     const T h6 = (T)(st->dt / 6.0);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        T v[3];
+    T v[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const long long j = c * N + i;
-            v[c] = m0[j] + h6 * (k1[j] + (T)2 * k2[j] + (T)2 * k3[j] + k4[j]);
-        }
-        const T n2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-        const T inv = n2 > (T)0 ? (T)1 / sqrt(n2) : (T)0;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) m0[c * N + i] = v[c] * inv;
+    for (int c = 0; c < 3; ++c) {
+        const long long j = c * N + i;
+        v[c] = m0[j] + h6 * (k1[j] + (T)2 * k2[j] + (T)2 * k3[j] + k4[j]);
     }
-    fixed_finish(st, tick);
+    const T n2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+    const T inv = n2 > (T)0 ? (T)1 / sqrt(n2) : (T)0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) m0[c * N + i] = v[c] * inv;
 }
 
 template <typename T>
@@ -381,7 +384,7 @@ static void rk4_step_t(mm_ctx* c) {
     const unsigned terms = c->terms;
     const bool demag = c->dm.on && (terms & MM_TERM_DEMAG);
     const long long N = c->N, n3 = 3 * N;
-    const unsigned tb = 256, nb3 = (unsigned)((n3 + tb - 1) / tb);
+    const unsigned tb = 256, nb3 = (unsigned)((n3 + tb - 1) / tb), nb = (unsigned)((N + tb - 1) / tb);
     static const double cs[4] = {0.0, 0.5, 0.5, 1.0};
     for (int s = 0; s < 4; ++s) {
         const void* ms = c->d_m;
@@ -395,9 +398,10 @@ static void rk4_step_t(mm_ctx* c) {
     }
     {
         LaunchScope ls(c, "rk4_final", (double)sizeof(T) * N * 18);
-        launch_dep(rk4_final_kernel<T>, counted_blocks(N, tb), tb, 0, c, c->d_state, (T*)c->d_m,
-                   (const T*)c->d_k[0], (const T*)c->d_k[1], (const T*)c->d_k[2], (const T*)c->d_k[3], N, c->d_tick);
+        launch_dep(rk4_final_kernel<T>, nb, tb, 0, c, c->d_state, (T*)c->d_m, (const T*)c->d_k[0],
+                   (const T*)c->d_k[1], (const T*)c->d_k[2], (const T*)c->d_k[3], N);
     }
+    step_next(c);
 }
 
 void rk4_step(mm_ctx* c) {
@@ -411,7 +415,8 @@ void heun_step(mm_ctx* c) {
     // predictor: k1 = f(m, H(m) + H_th); m* = m + dt k1
     demag_and_field(c, demag, MODE_HEUN1, terms, c->d_m, c->d_mtmp, c->d_k[0], nullptr, nullptr, 1, 0);
     // corrector: m' = normalise(m + dt/2 (k1 + f(m*, H(m*) + H_th))), same noise
-    demag_and_field(c, demag, MODE_HEUN2, terms, c->d_mtmp, c->d_m, nullptr, c->d_m, c->d_k[0], 1, 0, true);
+    demag_and_field(c, demag, MODE_HEUN2, terms, c->d_mtmp, c->d_m, nullptr, c->d_m, c->d_k[0], 1, 0);
+    step_next(c);
 }
 
 // Depondt-Mertens (Methods, "Integrators"): Omega_1 = Omega(m) and the
@@ -424,7 +429,8 @@ void dm_step(mm_ctx* c) {
     const unsigned terms = c->terms;
     const bool demag = c->dm.on && (terms & MM_TERM_DEMAG);
     demag_and_field(c, demag, MODE_DM1, terms, c->d_m, c->d_mtmp, c->d_k[0], nullptr, nullptr, 1, 0);
-    demag_and_field(c, demag, MODE_DM2, terms, c->d_mtmp, c->d_m, nullptr, c->d_m, c->d_k[0], 1, 0, true);
+    demag_and_field(c, demag, MODE_DM2, terms, c->d_mtmp, c->d_m, nullptr, c->d_m, c->d_k[0], 1, 0);
+    step_next(c);
 }
 
 // Adaptive Depondt-Mertens: err = max over cells |cand - m*| (the corrector
