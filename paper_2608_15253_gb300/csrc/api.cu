@@ -877,6 +877,13 @@ static void launch_attempts(mm_ctx* c, int n) {
     }
 }
 
+// n steps of a batch the way that mm_step runs them in the present launch shape
+static void launch_batch_steps(mm_ctx* c, int n) {
+    double t = c->h_state.t;
+    if (batch_is_fused(c->batch)) batch_macro_steps(c, c->batch, n, &t);
+    else launch_attempts(c, n);
+}
+
 static const int kChunk = 8;
 static const int kMacroBlock = 1024;   // steps per launch of the one-cell replica kernel
 
@@ -1427,9 +1434,9 @@ mm_status mm_batch_autotune(mm_ctx* c, const char* cache_path, int* nt_out, int*
                 c->h_state.target = std::numeric_limits<long long>::max();
                 c->h_state.t_end = std::numeric_limits<double>::infinity();
                 push_state(c);
-                launch_attempts(c, 1);     // warm-up
+                launch_batch_steps(c, 1);     // warm-up
                 cudaEventRecord(e0, c->stream);
-                launch_attempts(c, 3);
+                launch_batch_steps(c, 3);
                 cudaEventRecord(e1, c->stream);
                 cudaEventSynchronize(e1);
                 float ms = 0.f;
@@ -1439,7 +1446,8 @@ mm_status mm_batch_autotune(mm_ctx* c, const char* cache_path, int* nt_out, int*
             }
         }
         {
-            // the stacked shape: per size class, passes over all of its replicas
+            // the stacked shape: per size class, passes over all of its replicas, or
+            // blocks of steps of small films
             batch_set_shape(c->batch, 0, 0);
             int got_nt = -1, got_b = -1;
             batch_get_shape(c->batch, &got_nt, &got_b);
@@ -1447,9 +1455,9 @@ mm_status mm_batch_autotune(mm_ctx* c, const char* cache_path, int* nt_out, int*
                 c->h_state.target = std::numeric_limits<long long>::max();
                 c->h_state.t_end = std::numeric_limits<double>::infinity();
                 push_state(c);
-                launch_attempts(c, 1);
+                launch_batch_steps(c, 1);
                 cudaEventRecord(e0, c->stream);
-                launch_attempts(c, 3);
+                launch_batch_steps(c, 3);
                 cudaEventRecord(e1, c->stream);
                 cudaEventSynchronize(e1);
                 float ms = 0.f;

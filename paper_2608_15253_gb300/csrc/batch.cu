@@ -294,8 +294,8 @@ static void launch_stage(mm_ctx* c, BatchHost* b, int stage) {
     else batch_kernel_launch_256(a, b->blocks, b->smem, c->stream);
 }
 
-// Small films with demag are fused in the stacked shape, which the autotuner
-// picks for them; the persistent shape stays what the caller asked for.
+// Small films with demag are fused in the stacked shape, which the autotuner times
+// with them; the persistent shape stays what the caller asked for.
 bool batch_is_fused(BatchHost* b) { return b->macro || b->tile || (b->tile_demag && b->stacked); }
 
 // Ensembles with demag count their time step by step in every launch shape, t
@@ -559,7 +559,8 @@ void batch_get_shape(BatchHost* b, int* nt, int* blocks) {
 }
 
 
-// signature of the batch for the autotuner cache: sizes histogram + demag flag
+// signature of the batch for the autotuner cache: sizes histogram, terms, and
+// whether the stacked shape was timed with blocks of steps
 std::string batch_signature(BatchHost* b, unsigned terms) {
     std::vector<std::pair<long long, int>> h;
     for (const RepDev& r : b->rep) {
@@ -569,7 +570,7 @@ std::string batch_signature(BatchHost* b, unsigned terms) {
         if (!f) h.push_back({key, 1});
     }
     std::sort(h.begin(), h.end());
-    std::string s = "t" + std::to_string(terms);
+    std::string s = "t" + std::to_string(terms) + (b->tile_demag ? "b" : "");
     for (auto& e : h) s += "_" + std::to_string(e.first / 100000) + "x" + std::to_string(e.first % 100000) + "n" + std::to_string(e.second);
     return s;
 }

@@ -43,3 +43,27 @@ def test_a_run_to_a_time_steps_while_the_summed_time_is_below_it(shape, dt, t_en
         assert mm.mm_get_time(ctx) == (t, dt, n + 5)
     finally:
         mm.mm_destroy(ctx)
+
+
+@pytest.mark.parametrize("R", [4, 256])
+def test_the_autotuner_times_what_a_step_runs(R, tmp_path):
+    """The stacked shape runs blocks of steps of these films, 5 to 15 times as fast
+    as the per-class passes: the autotuner picks it, and the time that it records
+    is that of a step (within a factor of 3: three steps a launch, and the clock's
+    ramp)."""
+    mm = need_gpu()
+    import json
+    import time
+    ctx = _films(mm, 16, R, 1e-14)
+    try:
+        cache = tmp_path / "shapes"
+        assert mm.mm_batch_autotune(ctx, str(cache))[0] == 0
+        recorded = list(json.loads(cache.read_text().splitlines()[-1]).values())[0]
+        assert recorded["nt"] == 0
+        mm.mm_step(ctx, 1024)
+        t = time.perf_counter()
+        mm.mm_step(ctx, 1024)
+        step = 1e3 * (time.perf_counter() - t) / 1024
+        assert step / 3 < recorded["ms_per_step"] < 3 * step
+    finally:
+        mm.mm_destroy(ctx)
