@@ -46,6 +46,7 @@ struct BatchHost {
     bool macro = false;     // every replica one cell, no demag: macro_kernel
     bool tile = false;      // no demag, every replica at most kTileMaxCells cells: tile_kernel
     bool tile_demag = false;   // one small size class with demag: tile_demag_kernel in the stacked shape
+    bool thermal = false;   // the thermal term is on
     int nmax = 0;           // largest replica (cells)
     // retire/refill
     bool trials_on = false;
@@ -145,6 +146,7 @@ mm_status batch_setup(mm_ctx* c, BatchHost* b, const std::vector<mm_grid>& grids
             cudaMemcpy(k.d_members, k.members.data(), sizeof(int) * k.Rc, cudaMemcpyHostToDevice);
         }
     }
+    b->thermal = (c->terms & MM_TERM_THERMAL) != 0;
     b->macro = !demag;
     b->nmax = 0;
     for (const RepDev& d : b->rep) {
@@ -492,8 +494,14 @@ void batch_step(mm_ctx* c, BatchHost* b) {
 
 // nt = 0 selects the stacked launch shape (its per-class buffers are
 // allocated here, outside any graph capture; on failure the persistent
-// kernel stays)
+// kernel stays).  Blocks of steps keep their films on the SM and need none.  The
+// demag field's is allocated for classes whose fused kernel leaves it out as well:
+// a strain can turn further local terms on later, which that kernel does not have.
 void batch_set_shape(BatchHost* b, int nt, int blocks) {
+    if (nt == 0 && b->tile_demag) {
+        b->stacked = true;
+        return;
+    }
     if (nt == 0) {
         bool ok = true;
         for (size_t q = 0; q < b->ch.size() && ok; ++q) {
@@ -519,7 +527,7 @@ void batch_set_shape(BatchHost* b, int nt, int blocks) {
         if (ok) {
             for (ClassHost& k : b->ch) {
                 const size_t nb = sizeof(float) * (size_t)k.Rc * 3 * k.nx * k.ny;
-                if (!k.noise && cudaMalloc(&k.noise, nb) != cudaSuccess) {
+                if (b->thermal && !k.noise && cudaMalloc(&k.noise, nb) != cudaSuccess) {
                     k.noise = nullptr;
                     cudaGetLastError();
                 }

@@ -67,3 +67,26 @@ def test_the_autotuner_times_what_a_step_runs(R, tmp_path):
         assert step / 3 < recorded["ms_per_step"] < 3 * step
     finally:
         mm.mm_destroy(ctx)
+
+
+@pytest.mark.parametrize("n, terms, most", [(16, 0, 0.0), (40, 1 | 8 | 16, 1.0), (40, 0, 2.0)])
+def test_the_stacked_shape_allocates_what_its_kernels_read(n, terms, most):
+    """Blocks of steps need no buffer; the class passes need the spectra and the
+    demag field, and the thermal field of a step (12 bytes a cell) where that term is
+    on: `most` times 12 bytes a cell beside the spectra, and 4 MB for the modules."""
+    mm = need_gpu()
+    import torch
+    R = 4096
+    M = mm.Material(MAT.Ms, MAT.A, MAT.alpha, MAT.Ku1, MAT.u)
+    cfg = mm.make_config(precision=32, integrator=mm.MM_HEUN, demag=mm.MM_DEMAG_EXACT, dt=1e-14, terms=terms)
+    warm = _films(mm, n, 2, 1e-14)                  # (kernels loaded)
+    ctx = mm.mm_create_batch([mm.make_grid(n, n, 1, *CELL)] * R, M.s, cfg)
+    try:
+        free = torch.cuda.mem_get_info()[0]
+        mm.mm_batch_set_shape(ctx, 0)
+        taken = free - torch.cuda.mem_get_info()[0]
+        spectra = 0 if n == 16 else R * 3 * n * 52 * 8          # rows padded to 96: 49 columns, a pitch of 52
+        assert taken <= spectra + most * 12 * R * n * n + (4 << 20)
+    finally:
+        mm.mm_destroy(warm)
+        mm.mm_destroy(ctx)
