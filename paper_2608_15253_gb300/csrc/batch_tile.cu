@@ -10,9 +10,19 @@
 // in registers for both evaluations.  The stacked shape spends five launches of
 // 5 to 10 us on each evaluation of 256 films of 16x16, at a fifth of the chip's
 // warps; here an evaluation is six barriers: 64 Depondt-Mertens steps of those
-// films 2.4 -> 0.72 ms on one GB300 (11 us a step, bound by the chain of
+// films 4.7 -> 0.68 ms on one GB300 (10.6 us a step, bound by the chain of
 // phases in a CTA; 288 threads, which would take every phase in one round,
 // spill: 0.81 ms).
+//
+// Taken for every ensemble of one such size, whatever their number: against the
+// class passes of this library, us a Depondt-Mertens step at 300 K,
+//   films          64            256           1024          8192
+//   8x8        5.9 / 110     6.1 / 205    10.5 / 594     57 / 4132
+//   12x12     11.6 / 117    12.4 / 256    28.8 / 827    189 / 6027
+//   16x16      8.3 / 57     10.8 / 67     36.4 / 89     261 / 338
+//   24x24     13.5 / 58     25.3 / 72     87.0 / 131    673 / 721
+//   32x32     15.4 / 59     29.3 / 80      102 / 162    779 / 973
+// (two to eight of the smaller films share an SM, one of 24x24 or 32x32).
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -59,13 +59,13 @@ struct XArgs {
     const uint8_t* region;
     const Region<T>* lut;
     long long cells_per_comp;  // N: row r belongs to component r / (N/nx)
-    // fused RK stage (FP32 warp R2C, stage >= 1): the input rows are
+    // fused RK stage (stage >= 1): the input rows are
     // m_s = m0 + sum_j (dt a_sj) k_j, formed here and also written to ms
     const DevState* st;
     T* const* kptr;
     const T* m0;
     T* ms;
-    int stage;              // runtime stage for the CTA-wide R2C kernels (0: plain rows)
+    int stage;              // 0: plain rows
 };
 
 // m_s = m0 + sum_{j<S} (dt a_sj) k_j at element q (runtime stage S >= 1)

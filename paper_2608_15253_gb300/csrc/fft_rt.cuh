@@ -1,5 +1,6 @@
 // Runtime-planned in-shared-memory FFT (any length 2^a 3^b): the generic
-// path behind the compile-time specialised one in fft_ct.cuh.
+// path behind the register FFTs over lanes (fft_lane.cuh) and the compile-time
+// plans of the persistent batched kernel (fft_ct.cuh).
 #pragma once
 
 #include "common.cuh"

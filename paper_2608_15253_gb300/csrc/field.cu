@@ -137,7 +137,7 @@ static void field_launch_t(mm_ctx* c, int mode, unsigned terms, const T* m, cons
     const bool vec = sizeof(T) == 4 && c->uniform && !a.region && g.nx % kFieldV == 0 && a.R0.present != (T)0;
     const int gx = vec ? (g.nx / kFieldV + 31) / 32 : (g.nx + 31) / 32;
     int by = 8;
-    while (by > 1 && (long long)gx * ((g.ny + by - 1) / by) * g.nz < 4 * 152) by /= 2;
+    while (by > 1 && (long long)gx * ((g.ny + by - 1) / by) * g.nz < 4 * sm_count()) by /= 2;
     dim3 blk(32, by);
     dim3 grd(gx, (g.ny + by - 1) / by, g.nz);
     LaunchScope ls(c, kFieldNames[mode], field_bytes(c, mode, terms, Hd != nullptr));

@@ -1,7 +1,7 @@
 // Middle pass of 3-D grids (conv_lane.cuh, lane_conv_kernel): shapes by line
 // length.  One GB300, one evaluation:
-//   512x512x64 (L = 128)  551 us against 580 for one column per thread with
-//                         the components in turn; 3.7 TB/s of the 2.02 GB
+//   512x512x64 (L = 128)  570 us against 590 for one column per thread with
+//                         the components in turn; 3.5 TB/s of the 2.02 GB
 //   250x250x40 (L = 81)   111 us against 137
 //   150x150x24 (L = 48)   22.6 us against 26.7
 //   256x256x16 (L = 32)   30.4 us against 34.5 for whole lines in registers
@@ -9,7 +9,8 @@
 // of two columns (96 against 168) keep twice the warps on an SM, which hides
 // the exchange better than packed arithmetic shortens it (L = 48: 22.6
 // against 26.7 us).  At 128 points shared memory limits the warps, and two
-// columns per thread with the inputs prefetched win (551 against 628 us).
+// columns per thread with the inputs prefetched win (551 against 628 us by
+// themselves, 570 in a step).
 #include "conv_lane.cuh"
 #include "lane.h"
 

@@ -4,9 +4,10 @@
 // counted through all films of the class.  One GB300, five classes of the
 // 1024-replica ensemble, mean of a class: predictor 41.0 us, corrector 36.3
 // against 15.3 for the inverse X pass and 31.9 / 26.9 for the field kernel.
-// What bounds it is issue: some 700 instructions a cell, a third of them the
-// thermal draw.  Rows of four cells a thread only (16-byte accesses), films of
-// up to 256 columns.
+// What bounds it: 520 instructions a cell in the predictor, the thermal draw among
+// them, 340 in the corrector, and their loads; half of the issue slots are taken at
+// the 12 warps an SM that 128 registers allow.  Rows of four cells a thread only
+// (16-byte accesses), films of up to 256 columns.
 #pragma once
 
 #include <cuda_runtime.h>
